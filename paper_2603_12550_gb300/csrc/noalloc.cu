@@ -36,7 +36,7 @@ constexpr size_t kRecBytes =
     (size_t)((VDS_NOALLOC_MAX_N + vds_pair::TJ - 1) / vds_pair::TJ * vds_pair::TJ) * kMaxDP * sizeof(float);
 constexpr size_t kPartBytes = (size_t)4 << 20;
 constexpr size_t kScratchBytes = kHeadBytes + kRecBytes + kPartBytes;
-static_assert(kRedOff + (VDS_NOALLOC_MAX_N / 256 + 1) * 4 * 8 <= kHeadBytes, "head layout");
+static_assert(kRedOff + (VDS_NOALLOC_MAX_N / 32 + 1) * 8 <= kHeadBytes, "head layout: one energy partial per CTA");
 
 }  // namespace
 
@@ -85,7 +85,7 @@ int setup_device(int dev, DevState **out) {
 // the partial sums fit; without it a shape whose partials do not fit at the
 // full grid is declined (done = false, nothing launched).
 template <int D, int RI, int NT, bool GRAD, int TJK>
-int na_try(const DevState &s, int N, cudaStream_t st, const float *rec, double *part, int *err,
+int na_try(const DevState &s, int N, cudaStream_t st, const float *rec, float2 *part, int *err,
            Sched &sc, bool shrink, bool &done) {
   using namespace vds_pair;
   static_assert(Rec<D>::DP <= kMaxDP, "record area sized for the widest D");
@@ -103,20 +103,15 @@ int na_try(const DevState &s, int N, cudaStream_t st, const float *rec, double *
   sc.Npad = (N + TJ - 1) / TJ * TJ;
   sc.Nipad = sc.Npad;
   sc.nchunk = sc.Npad / TJK;
+  sc.cpt = 0;
   sc.n_itiles = (N + TI - 1) / TI;
   sc.items = (long long)sc.n_itiles * sc.nchunk;
   long long G = (long long)s.num_sms * occ;
   if (G > sc.items) G = sc.items;
   for (;;) {
     sc.G = (int)G;
-    int maxseg = 1;
-    for (int t = 0; t < sc.n_itiles; ++t) {
-      const int f = sched_first_cta((long long)t * sc.nchunk, sc);
-      const int l = sched_first_cta((long long)(t + 1) * sc.nchunk - 1, sc);
-      if (l - f + 1 > maxseg) maxseg = l - f + 1;
-    }
-    sc.maxseg = maxseg;
-    if ((size_t)sc.n_itiles * maxseg * TI * ACC * sizeof(double) <= kPartBytes) break;
+    sc.maxseg = sched_maxseg(sc);
+    if ((size_t)sc.n_itiles * sc.maxseg * TI * ACC * sizeof(float2) <= kPartBytes) break;
     if (!shrink) return VDS_OK;
     if (G == 1) return VDS_ESIZE;
     G = G * 3 / 4;
@@ -132,7 +127,7 @@ int na_try(const DevState &s, int N, cudaStream_t st, const float *rec, double *
 // half the SMs' worth of items, 64-record j-chunks below 8 items per SM if
 // their partials fit, otherwise 256-record j-chunks).
 template <int D, bool GRAD>
-int na_pair(const DevState &s, int N, cudaStream_t st, const float *rec, double *part, int *err,
+int na_pair(const DevState &s, int N, cudaStream_t st, const float *rec, float2 *part, int *err,
             Sched &sc) {
   using namespace vds_pair;
   constexpr int RI = GRAD ? PairCfg<D>::RI_GRAD : PairCfg<D>::RI_DENS;
@@ -158,24 +153,23 @@ int na_energy_grad(const DevState &s, const float *q, const KParams &kp, double 
   double *scal = (double *)(base + kScalOff);
   double *red = (double *)(base + kRedOff);
   float *rec = (float *)(base + kHeadBytes);
-  double *part = (double *)(base + kHeadBytes + kRecBytes);
+  float2 *part = (float2 *)(base + kHeadBytes + kRecBytes);
   const int N = kp.N;
   const int Npad = (N + TJ - 1) / TJ * TJ;
   // error flag and tickets must start at zero
   VDS_CUDA_TRY(cudaMemsetAsync(base, 0, kScalOff, st));
   k_prep<D><<<(Npad + 255) / 256, 256, 0, st>>>(N, Npad, kp.c, q, nullptr, nullptr, 0.f, nullptr, rec);
   VDS_CUDA_TRY(cudaGetLastError());
-  Sched sd, sg;
-  VDS_TRY((na_pair<D, false>(s, N, st, rec, part, err, sd)));
-  const int nb = (N + NT_FIN - 1) / NT_FIN;
-  k_dens_finish<D><<<nb, NT_FIN, 0, st>>>(sd, part, rec, rho, kp, E ? 1 : 0, q, nullptr, nullptr, nullptr,
-                                         red, ticket + TK_DENS, scal, err);
-  VDS_CUDA_TRY(cudaGetLastError());
+  PartSrc src;
+  src.i = part;
+  src.j = nullptr;
+  VDS_TRY((na_pair<D, false>(s, N, st, rec, part, err, src.sc)));
+  const FinArgs ad{rec, rho, q, nullptr, nullptr, nullptr, nullptr, E ? 1 : 0, red, ticket + TK_DENS, scal, err};
+  VDS_TRY((launch_dens_finish<D>(st, src, kp, ad)));
   if (g) {
-    VDS_TRY((na_pair<D, true>(s, N, st, rec, part, err, sg)));
-    k_grad_finish<D, GM_OUT><<<nb, NT_FIN, 0, st>>>(sg, part, rec, kp, g, q, nullptr, nullptr, nullptr,
-                                                   nullptr, red, ticket + TK_GRAD, scal, err);
-    VDS_CUDA_TRY(cudaGetLastError());
+    VDS_TRY((na_pair<D, true>(s, N, st, rec, part, err, src.sc)));
+    const FinArgs ag{rec, g, q, nullptr, nullptr, nullptr, nullptr, 0, red, ticket + TK_GRAD, scal, err};
+    VDS_TRY((launch_grad_finish<D, GM_OUT>(st, src, kp, ag)));
   }
   double e_host = 0.0;
   int err_host = 0;

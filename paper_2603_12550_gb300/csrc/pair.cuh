@@ -7,12 +7,16 @@
 // pair square, flattened i-tile major, are split into G contiguous equal
 // ranges, one per CTA of a grid sized to the resident capacity of the GPU.
 // A CTA accumulates in registers while its i-tile is unchanged and writes one
-// FP64 partial per (i-tile, segment); an epilogue sums the segments of each
-// i-tile in a fixed order, so results do not depend on timing.
+// partial (an FP32 sum and its compensation) per (i-tile, segment, component);
+// an epilogue sums the segments of each i-tile in a fixed order, so results do
+// not depend on timing.
+// With cpt > 0 (the symmetric passes) i-tile t takes the j-chunks from its
+// own first one on, cpt per tile: the upper triangle of the square.
 struct Sched {
-  long long items;  // n_itiles * nchunk
+  long long items;  // sched_start(n_itiles)
   int G;            // CTAs
-  int nchunk;       // j-chunks (tiles of TJ records) per i-tile
+  int nchunk;       // j-chunks
+  int cpt;          // j-chunks per i-tile left out below the diagonal (0: none)
   int n_itiles;
   int maxseg;       // max segments per i-tile
   int TI;           // particles per i-tile
@@ -23,6 +27,21 @@ struct Sched {
 
 __host__ __device__ __forceinline__ int sched_first_cta(long long x, const Sched &s) {
   return (int)(((x + 1) * (long long)s.G + s.items - 1) / s.items - 1);
+}
+
+// First item of i-tile t (t <= n_itiles).
+__host__ __device__ __forceinline__ long long sched_start(int t, const Sched &s) {
+  return (long long)t * s.nchunk - (long long)s.cpt * ((long long)t * (t - 1) / 2);
+}
+
+// Symmetric passes: partials of the j side, one row of sums per i-tile t
+// and component over the particles of the tiles after it, [t][component][j -
+// (t + 1) TI].  Columns of row t, and the row's first element per component.
+__host__ __device__ __forceinline__ long long sched_jcols(int t, const Sched &s) {
+  return (long long)(s.nchunk - (t + 1) * s.cpt) * (s.TI / s.cpt);
+}
+__host__ __device__ __forceinline__ long long sched_jrow(int t, const Sched &s) {
+  return ((long long)t * s.nchunk - (long long)s.cpt * ((long long)t * (t + 1) / 2)) * (s.TI / s.cpt);
 }
 
 // Physical parameters as the kernels see them.
@@ -53,13 +72,9 @@ int pass_prep(vds_ctx *c, const KParams &kp, const float *base, const float *del
 //   (1/N) sum_I [kBT (ln rho_I + lnorm) + Psi(y_I)]
 //   + (zeta/2dt)(1/N) sum_I dI^T (A^-1 (x) I) dI,   dI = qa_I - qb_I
 // (the quadratic term only when qa != NULL; qb may be NULL) into scal[SC_E].
-// y_I = ybase_I + ydelta_I (ydelta may be NULL).  expand: large clouds take
-// the squared distances through the records' norms (D + 2 instead of 2D + 1
-// FP32 operations per pair; 1e-6 relative in the kernel values), for the
-// reduced model's refresh cycle; the records must come from pass_prep.
+// y_I = ybase_I + ydelta_I (ydelta may be NULL).
 int pass_density(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
-                 const float *ybase, const float *ydelta, const float *qa,
-                 const float *qb, bool expand = false);
+                 const float *ybase, const float *ydelta, const float *qa, const float *qb);
 
 // The same density without the energy, with the pair dot products on the
 // tensor cores (dens_tc.cu: 3xTF32; 1e-5 relative for the median particle of

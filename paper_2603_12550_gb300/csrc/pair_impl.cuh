@@ -2,6 +2,10 @@
 // pair_impl.cuh -- the O(N^2) Gaussian-kernel pair passes of the VDS hot path and
 // their fused O(N) epilogues, for GB300 (sm_103a).
 //
+// k_pair is the ordered form (rows of any points against all particles): the
+// queries, the row ranges and the allocation-free evaluation; a cloud against
+// itself takes the symmetric form of pair_sym.cuh from SYM_MIN_N particles on.
+//
 // Density pass (Eq. model_DeteParAppr, denominators of Eq. model_DymRepPar):
 //   rho_I = sum_J exp2(-|qhat_I - qhat_J|^2),  qhat = c q,  c^2 = log2(e)/(2h^2)
 // Gradient pass (Eq. model_DymRepPar with grad K = -(x/h^2) K):
@@ -17,6 +21,8 @@
 #include <math.h>
 
 #include "pair.cuh"
+#include "pair_fin.cuh"
+#include "pair_sym.cuh"
 
 namespace vds_pair {
 
@@ -53,22 +59,17 @@ constexpr int NT_SMALL = 128, RI_SMALL = 1, TJ_SMALL = 64;
 
 // ------------------------------------------------------------- pair kernel
 
-// EXP (density pass only, records with their squared norm in slot D + 1):
-// the squared distance through the norms, |x|^2 + |y|^2 - 2 x.y, D + 2 FP32
-// operations per pair instead of 2D + 1, with an absolute error of a few
-// units of FP32 rounding of |x|^2 + |y|^2 (1e-6 relative in the kernel value
-// for the bulk of a cloud).  Only the reduced model's refresh cycle takes
-// it; the full-order path keeps the differences its 1e-5 bar needs.
+// Records with a norm slot (D + 1): the squared norm of qhat, for the passes
+// that form their dot products on the tensor cores.
 template <int D>
 struct HasNorm {
   static constexpr bool value = Rec<D>::DP >= D + 2;
 };
 
-template <int D, int RI, int NT, bool GRAD, int TJK = TJ, bool EXP = false>
+template <int D, int RI, int NT, bool GRAD, int TJK = TJ>
 __global__ void __launch_bounds__(NT)
     k_pair(const float *__restrict__ rec, const float *__restrict__ reci, Sched sc,
-           double *__restrict__ part, int *__restrict__ err) {
-  static_assert(!EXP || (!GRAD && HasNorm<D>::value), "expanded distances: density pass, norm slot");
+           float2 *__restrict__ part, int *__restrict__ err) {
   static_assert(TJ % TJK == 0, "j-tiles divide the record padding");
   constexpr int DP = Rec<D>::DP;
   constexpr int ACC = GRAD ? D : 1;
@@ -98,7 +99,6 @@ __global__ void __launch_bounds__(NT)
 
   float xi[RI][D];
   float wi[RI];
-  float ni[RI];
   float sum[RI][ACC], cmp[RI][ACC];
   int cur = -1, seg = 0;
   long long it_fail = -1;
@@ -107,9 +107,10 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
     for (int k = 0; k < RI; ++k) {
       const int il = tid + k * NT;
-      double *dst = part + (((size_t)cur * sc.maxseg + seg) * sc.TI + il) * ACC;
 #pragma unroll
-      for (int a = 0; a < ACC; ++a) dst[a] = (double)sum[k][a] - (double)cmp[k][a];
+      for (int a = 0; a < ACC; ++a)
+        part[(((size_t)cur * sc.maxseg + seg) * ACC + a) * sc.TI + il] =
+            make_float2(sum[k][a], -cmp[k][a]);
     }
   };
 
@@ -127,7 +128,6 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
         for (int d = 0; d < D; ++d) xi[k][d] = r[d];
         wi[k] = GRAD ? r[D] : 0.f;
-        ni[k] = EXP ? r[D + 1] : 0.f;
 #pragma unroll
         for (int a = 0; a < ACC; ++a) sum[k][a] = cmp[k][a] = 0.f;
       }
@@ -162,20 +162,12 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
       for (int k = 0; k < RI; ++k) {
         float dd[D];
-        float r2;
-        if constexpr (EXP) {
-          float dot = xi[k][0] * xj[0];
+        dd[0] = xi[k][0] - xj[0];
+        float r2 = dd[0] * dd[0];
 #pragma unroll
-          for (int d = 1; d < D; ++d) dot = fmaf(xi[k][d], xj[d], dot);
-          r2 = fmaf(-2.f, dot, ni[k] + xj[(D + 1) % DP]);
-        } else {
-          dd[0] = xi[k][0] - xj[0];
-          r2 = dd[0] * dd[0];
-#pragma unroll
-          for (int d = 1; d < D; ++d) {
-            dd[d] = xi[k][d] - xj[d];
-            r2 = fmaf(dd[d], dd[d], r2);
-          }
+        for (int d = 1; d < D; ++d) {
+          dd[d] = xi[k][d] - xj[d];
+          r2 = fmaf(dd[d], dd[d], r2);
         }
         const float e = ex2_approx(-r2);
         if constexpr (!GRAD) {
@@ -220,46 +212,6 @@ __global__ void __launch_bounds__(NT)
   if (cur >= 0) flush();
 }
 
-// --------------------------------------------------------- small device math
-
-__device__ __forceinline__ double rouse_A(int j, int k) {
-  return j == k ? 2.0 : ((j - k == 1 || k - j == 1) ? -1.0 : 0.0);
-}
-
-// inverse of the tridiagonal Rouse matrix: min(j,k)(nb+1-max(j,k))/(nb+1), 1-based
-__device__ __forceinline__ double rouse_Ainv(int j, int k, int nb) {
-  const int lo = (j < k ? j : k) + 1, hi = (j > k ? j : k) + 1;
-  return (double)lo * (double)(nb + 1 - hi) / (double)(nb + 1);
-}
-
-// Spring energy and force factor per bond: grad Psi_k = f_k q_k.
-template <int D>
-__device__ __forceinline__ bool spring_eval(const KParams &kp, const double (&y)[D], double &psi,
-                                            double (&f)[8]) {
-  psi = 0.0;
-  bool ok = true;
-  for (int k = 0; k < kp.nb; ++k) {
-    double n2 = 0.0;
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-      if (a / kp.s == k) n2 += y[a] * y[a];
-    if (kp.spring == 0) {
-      psi += 0.5 * kp.H[k] * n2;
-      f[k] = kp.H[k];
-    } else {
-      const double x = 1.0 - n2 / kp.b;
-      if (!(x > 0.0)) {
-        ok = false;
-        f[k] = 0.0;
-      } else {
-        psi += -0.5 * kp.H[k] * kp.b * log(x);
-        f[k] = kp.H[k] / x;
-      }
-    }
-  }
-  return ok;
-}
-
 // --------------------------------------------------------------- prep kernel
 
 template <int D>
@@ -297,251 +249,6 @@ __global__ void k_prep(int N, int Npad, float c, const float *__restrict__ base,
   float4 *dst = reinterpret_cast<float4 *>(rec + (size_t)i * DP);
 #pragma unroll
   for (int v = 0; v < DP / 4; ++v) dst[v] = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
-}
-
-// ------------------------------------------------------------- epilogues
-
-constexpr int NT_FIN = 256;
-
-// Deterministic grid reduction: every block stores its partial, the last
-// block to arrive (ticket) sums them in block order.  Returns true in the
-// thread that holds the final value.
-template <int K>
-__device__ __forceinline__ bool grid_reduce(double (&v)[K], const bool (&is_max)[K], double *red,
-                                            unsigned *ticket, double (&out)[K]) {
-  __shared__ double sh[NT_FIN / 32][K];
-  __shared__ bool last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double x = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double y = __shfl_xor_sync(0xffffffffu, x, o);
-      x = is_max[k] ? fmax(x, y) : x + y;
-    }
-    if (lane == 0) sh[w][k] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double x = is_max[k] ? 0.0 : 0.0;
-      for (int q = 0; q < NT_FIN / 32; ++q) x = is_max[k] ? fmax(x, sh[q][k]) : x + sh[q][k];
-      red[(size_t)blockIdx.x * K + k] = x;
-    }
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return false;
-  __threadfence();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double x = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) {
-      const double y = __ldcg(red + (size_t)b * K + k);
-      x = is_max[k] ? fmax(x, y) : x + y;
-    }
-    out[k] = x;
-  }
-  *ticket = 0u;
-  return true;
-}
-
-template <int D>
-__device__ __forceinline__ void load_y(const float *ybase, const float *ydelta, int i, double (&y)[D],
-                                       float (&yf)[D]) {
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    float v = ybase[(size_t)i * D + d];
-    if (ydelta) v = v + ydelta[(size_t)i * D + d];
-    yf[d] = v;
-    y[d] = (double)v;
-  }
-}
-
-template <int D>
-__global__ void __launch_bounds__(NT_FIN)
-    k_dens_finish(Sched sc, const double *__restrict__ part, float *__restrict__ rec,
-                  float *__restrict__ rho_out, KParams kp, int want_energy,
-                  const float *__restrict__ ybase, const float *__restrict__ ydelta,
-                  const float *__restrict__ qa, const float *__restrict__ qb, double *red,
-                  unsigned *ticket, double *scal, int *err) {
-  constexpr int DP = Rec<D>::DP;
-  const int i = blockIdx.x * NT_FIN + threadIdx.x;
-  double e = 0.0;
-  if (i < kp.N) {
-    const int t = i / sc.TI, il = i - t * sc.TI;
-    const int f = sched_first_cta((long long)t * sc.nchunk, sc);
-    const int l = sched_first_cta((long long)(t + 1) * sc.nchunk - 1, sc);
-    double rho = 0.0;
-    for (int g = 0; g <= l - f; ++g) rho += part[((size_t)t * sc.maxseg + g) * sc.TI + il];
-    if (!(rho >= 0.5 && rho <= 1e300)) vds_flag(err, VDS_ENAN);
-    rec[(size_t)i * DP + D] = (float)(1.0 / rho);
-    if (rho_out) rho_out[i] = (float)rho;
-    if (want_energy) {
-      double y[D];
-      float yf[D];
-      load_y<D>(ybase, ydelta, i, y, yf);
-      double psi, fk[8];
-      if (!spring_eval<D>(kp, y, psi, fk)) vds_flag(err, VDS_EDOMAIN);
-      e = kp.kBT * (log(rho) + kp.lnorm) + psi;
-      if (qa) {
-        double dl[D];
-#pragma unroll
-        for (int d = 0; d < D; ++d)
-          dl[d] = (double)qa[(size_t)i * D + d] - (qb ? (double)qb[(size_t)i * D + d] : 0.0);
-        double quad = 0.0;
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-#pragma unroll
-          for (int b = 0; b < D; ++b)
-            if (a % kp.s == b % kp.s) quad += dl[a] * rouse_Ainv(a / kp.s, b / kp.s, kp.nb) * dl[b];
-        e += kp.zeta / (2.0 * kp.dt) * quad;
-      }
-    }
-  }
-  if (want_energy) {
-    double v[1] = {e}, out[1];
-    const bool mx[1] = {false};
-    if (grid_reduce<1>(v, mx, red, ticket, out)) {
-      scal[SC_E] = out[0] / (double)kp.N;
-      if (!(fabs(scal[SC_E]) <= 1e300)) vds_flag(err, VDS_ENAN);
-    }
-  }
-}
-
-template <int D, int MODE>
-__global__ void __launch_bounds__(NT_FIN)
-    k_grad_finish(Sched sc, const double *__restrict__ part, float *__restrict__ rec, KParams kp,
-                  float *__restrict__ out, const float *ybase,
-                  const float *__restrict__ ydelta, const float *__restrict__ qa,
-                  const float *__restrict__ qb, float *q_io, double *red,
-                  unsigned *ticket, double *scal, int *err) {
-  constexpr int DP = Rec<D>::DP;
-  const int i = blockIdx.x * NT_FIN + threadIdx.x;
-  double dec = 0.0, dmax = 0.0, ymax = 0.0;
-  if (i < kp.N) {
-    const int t = i / sc.TI, il = i - t * sc.TI;
-    const int f = sched_first_cta((long long)t * sc.nchunk, sc);
-    const int l = sched_first_cta((long long)(t + 1) * sc.nchunk - 1, sc);
-    double g[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) g[a] = 0.0;
-    for (int s = 0; s <= l - f; ++s) {
-      const double *p = part + (((size_t)t * sc.maxseg + s) * sc.TI + il) * D;
-#pragma unroll
-      for (int a = 0; a < D; ++a) g[a] += p[a];
-    }
-    double y[D];
-    float yf[D];
-    load_y<D>(ybase, ydelta, i, y, yf);
-    double psi, fk[8];
-    if (!spring_eval<D>(kp, y, psi, fk)) vds_flag(err, VDS_EDOMAIN);
-#pragma unroll
-    for (int a = 0; a < D; ++a) g[a] = kp.kBT * (-kp.sfac * g[a]) + fk[a / kp.s] * y[a];
-
-    if constexpr (MODE == GM_OUT) {
-      if (qa) {
-        double dl[D];
-#pragma unroll
-        for (int d = 0; d < D; ++d)
-          dl[d] = (double)qa[(size_t)i * D + d] - (qb ? (double)qb[(size_t)i * D + d] : 0.0);
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          double v = 0.0;
-#pragma unroll
-          for (int b = 0; b < D; ++b)
-            if (a % kp.s == b % kp.s) v += rouse_Ainv(a / kp.s, b / kp.s, kp.nb) * dl[b];
-          g[a] += kp.zeta / kp.dt * v;
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < D; ++a) out[(size_t)i * D + a] = (float)g[a];
-    } else if constexpr (MODE == GM_VEL) {
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const int k = a / kp.s, al = a - k * kp.s;
-        double v = 0.0, m = 0.0;
-#pragma unroll
-        for (int b = 0; b < D; ++b) {
-          const int kb = b / kp.s, be = b - kb * kp.s;
-          if (kb == k) v += kp.kappa[al * kp.s + be] * y[b];
-          if (be == al) m += rouse_A(k, kb) * g[b];
-        }
-        out[(size_t)i * D + a] = (float)(v - m / kp.zeta);
-      }
-    } else if constexpr (MODE == GM_EXPLICIT) {
-      float yn[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const int k = a / kp.s, al = a - k * kp.s;
-        double v = 0.0, m = 0.0;
-#pragma unroll
-        for (int b = 0; b < D; ++b) {
-          const int kb = b / kp.s, be = b - kb * kp.s;
-          if (kb == k) v += kp.kappa[al * kp.s + be] * y[b];
-          if (be == al) m += rouse_A(k, kb) * g[b];
-        }
-        yn[a] = (float)(y[a] + kp.dt * (v - m / kp.zeta));
-      }
-      if (kp.spring == 1) {
-        for (int k = 0; k < kp.nb; ++k) {
-          double n2 = 0.0;
-#pragma unroll
-          for (int a = 0; a < D; ++a)
-            if (a / kp.s == k) n2 += (double)yn[a] * yn[a];
-          if (!(n2 < kp.b)) vds_flag(err, VDS_EDOMAIN);
-        }
-      }
-      float o[DP];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        q_io[(size_t)i * D + a] = yn[a];
-        o[a] = kp.c * yn[a];
-      }
-#pragma unroll
-      for (int a = D; a < DP; ++a) o[a] = 0.f;
-      float4 *dst = reinterpret_cast<float4 *>(rec + (size_t)i * DP);
-#pragma unroll
-      for (int v = 0; v < DP / 4; ++v) dst[v] = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
-    } else {  // GM_IMPLICIT_DIR
-      double dl[D];
-#pragma unroll
-      for (int d = 0; d < D; ++d) dl[d] = (double)ydelta[(size_t)i * D + d];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const int k = a / kp.s, al = a - k * kp.s;
-        double ag = 0.0, aid = 0.0;
-#pragma unroll
-        for (int b = 0; b < D; ++b) {
-          const int kb = b / kp.s, be = b - kb * kp.s;
-          if (be == al) {
-            ag += rouse_A(k, kb) * g[b];
-            aid += rouse_Ainv(k, kb, kp.nb) * dl[b];
-          }
-        }
-        const double dr = dl[a] + kp.dt / kp.zeta * ag;
-        const double G = kp.zeta / kp.dt * aid + g[a];
-        const float drf = (float)dr;
-        out[(size_t)i * D + a] = drf;
-        dec += G * dr;
-        dmax = fmax(dmax, fabs((double)drf));
-        ymax = fmax(ymax, fabs((double)yf[a]));
-      }
-    }
-  }
-  if constexpr (MODE == GM_IMPLICIT_DIR) {
-    double v[3] = {dec, dmax, ymax}, o[3];
-    const bool mx[3] = {false, true, true};
-    if (grid_reduce<3>(v, mx, red, ticket, o)) {
-      scal[SC_DEC] = o[0] / (double)kp.N;
-      scal[SC_DMAX] = o[1];
-      scal[SC_YMAX] = o[2];
-      if (!(fabs(o[0]) <= 1e300)) vds_flag(err, VDS_ENAN);
-    }
-  }
 }
 
 // ------------------------------------------------------------ stress kernel
@@ -638,9 +345,20 @@ __global__ void k_flow(KParams kp, const float *__restrict__ q, float *__restric
 
 // ------------------------------------------------------------ host plumbing
 
+// Most CTAs that share one i-tile.
+inline int sched_maxseg(const Sched &sc) {
+  int m = 1;
+  for (int t = 0; t < sc.n_itiles; ++t) {
+    const int f = sched_first_cta(sched_start(t, sc), sc);
+    const int l = sched_first_cta(sched_start(t + 1, sc) - 1, sc);
+    if (l - f + 1 > m) m = l - f + 1;
+  }
+  return m;
+}
+
 // i points: the Ni records at reci (the particles themselves unless a query
 // pass); j points: the N particle records in c->rec.
-template <int D, int RI, int NT, bool GRAD, int TJK = TJ, bool EXP = false>
+template <int D, int RI, int NT, bool GRAD, int TJK = TJ>
 int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
   constexpr int DP = Rec<D>::DP;
   constexpr int ACC = GRAD ? D : 1;
@@ -651,32 +369,27 @@ int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
   int &occ = occ_dev[c->device < VDS_MAX_DEVICES ? c->device : 0];
   if (occ <= 0 || c->device >= VDS_MAX_DEVICES) {
     // large D needs more than the default 48 KB of dynamic shared memory
-    VDS_CUDA_TRY(cudaFuncSetAttribute(k_pair<D, RI, NT, GRAD, TJK, EXP>,
+    VDS_CUDA_TRY(cudaFuncSetAttribute(k_pair<D, RI, NT, GRAD, TJK>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int o = 0;
-    VDS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_pair<D, RI, NT, GRAD, TJK, EXP>, NT, smem));
+    VDS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_pair<D, RI, NT, GRAD, TJK>, NT, smem));
     occ = o > 0 ? o : 1;
   }
   sc.TI = TI;
   sc.Npad = (N + TJ - 1) / TJ * TJ;
   sc.Nipad = (Ni + TJ - 1) / TJ * TJ;
   sc.nchunk = sc.Npad / TJK;
+  sc.cpt = 0;
   sc.n_itiles = (Ni + TI - 1) / TI;
   sc.items = (long long)sc.n_itiles * sc.nchunk;
   const long long cap = (long long)c->num_sms * occ;
   sc.G = (int)(sc.items < cap ? sc.items : cap);
-  int maxseg = 1;
-  for (int t = 0; t < sc.n_itiles; ++t) {
-    const int f = sched_first_cta((long long)t * sc.nchunk, sc);
-    const int l = sched_first_cta((long long)(t + 1) * sc.nchunk - 1, sc);
-    if (l - f + 1 > maxseg) maxseg = l - f + 1;
-  }
-  sc.maxseg = maxseg;
-  VDS_TRY(vds_ensure(c, c->part, (size_t)sc.n_itiles * maxseg * TI * ACC * sizeof(double)));
+  sc.maxseg = sched_maxseg(sc);
+  VDS_TRY(vds_ensure(c, c->part, (size_t)sc.n_itiles * sc.maxseg * TI * ACC * sizeof(float2)));
   const int pk = GRAD ? PK_GRADIENT : PK_DENSITY;
   VDS_TRY(vds_time_begin(c, pk));
-  k_pair<D, RI, NT, GRAD, TJK, EXP><<<sc.G, NT, smem, c->stream>>>((const float *)c->rec.ptr, reci, sc,
-                                                                     (double *)c->part.ptr, c->err);
+  k_pair<D, RI, NT, GRAD, TJK><<<sc.G, NT, smem, c->stream>>>((const float *)c->rec.ptr, reci, sc,
+                                                                     (float2 *)c->part.ptr, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
   VDS_TRY(vds_time_end(c, pk));
   ++c->launches;
@@ -701,34 +414,156 @@ int prep_impl(vds_ctx *c, const KParams &kp, const float *base, const float *del
 // four times the items, so that the last round of the stream-K split is
 // not a large fraction of the pass (N = 10000 at D = 9: 200 and 360 items
 // per pass at 256 records).
-// EXP: the expanded distances of the density pass, for large clouds only
-// (small clouds keep the direct form: their passes are latency bound).
-template <int D, bool GRAD, bool EXP = false>
+template <int D, bool GRAD>
 int launch_pass(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
   constexpr int RI = GRAD ? PairCfg<D>::RI_GRAD : PairCfg<D>::RI_DENS;
   constexpr int NT = GRAD ? PairCfg<D>::NT_GRAD : PairCfg<D>::NT_DENS;
   const long long items = (long long)((Ni + NT * RI - 1) / (NT * RI)) * ((N + TJ - 1) / TJ);
   if (2 * items < c->num_sms) return launch_pair<D, RI_SMALL, NT_SMALL, GRAD, TJ_SMALL>(c, N, sc, Ni, reci);
   if (items < 8LL * c->num_sms) return launch_pair<D, RI, NT, GRAD, TJ_SMALL>(c, N, sc, Ni, reci);
-  if constexpr (EXP && !GRAD && HasNorm<D>::value) return launch_pair<D, RI, NT, GRAD, TJ, true>(c, N, sc, Ni, reci);
-  else return launch_pair<D, RI, NT, GRAD>(c, N, sc, Ni, reci);
+  return launch_pair<D, RI, NT, GRAD>(c, N, sc, Ni, reci);
+}
+
+// Shapes of the symmetric passes, from sweeps of particles per lane (RI),
+// CTAs of 128 threads per SM (MINB: the register budget) and threads per CTA
+// on GB300: the most particles per lane whose warps still fill the schedulers.
+// Gradient, N = 65536, D = 9: RI = 6 at three CTAs 2.81 ms, 5 at three 2.95,
+// 4 at four 3.18, 8 at two 3.20 (k_pair 3.86).  D = 6: 8 at three 2.10, 6 at
+// four 2.12.  Density, D = 9: 10 at three 1.36, 8 at four 1.49, 12 at two 1.42
+// (k_pair 2.46).
+template <int D, bool GRAD>
+struct SymCfg {
+  static constexpr int RI = GRAD ? (D == 2 ? 12 : D <= 6 ? 8 : D <= 9 ? 6 : D == 12 ? 5 : 4)
+                                 : (D <= 4 ? 12 : D == 9 ? 10 : D <= 12 ? 8 : 4);
+  static constexpr int MINB128 = GRAD ? (D <= 4 ? 4 : D <= 10 ? 3 : 2) : (D == 9 || D == 12 ? 3 : 4);
+  static constexpr int NT_LARGE = MINB128 * 128;  // one CTA per SM
+};
+
+// The j sums of a symmetric pass may take this much workspace; larger clouds
+// (and a workspace that cannot be had) take the ordered form.
+constexpr size_t SYM_MAX_PARTJ = (size_t)4 << 30;
+constexpr int SYM_MIN_N = 2048;
+// From here on the gradient pass takes one CTA per SM: a third of the i-tiles
+// and of the j sums written and read (N = 65536, D = 9: 65 instead of 199 MB).
+constexpr int SYM_LARGE_N = 49152;
+// j-chunks of 64 records in the density pass from here on; 32 below, where the
+// items per CTA are few.
+constexpr int SYM_CHUNK_N = 32768;
+
+// The symmetric pass over the N records at c->rec; done = false (and nothing
+// launched) where its workspace is over the limit or cannot be had.
+template <int D, bool GRAD, int NT, int TJS>
+int launch_sym(vds_ctx *c, int N, Sched &sc, bool &done) {
+  using C = SymCfg<D, GRAD>;
+  constexpr int RI = C::RI, TI = NT * RI, ACC = GRAD ? D : 1, MINB = C::MINB128 * 128 / NT;
+  constexpr size_t smem = SymSmem<D, RI, NT, GRAD, TJS>::BYTES;
+  auto kern = k_sym<D, RI, NT, MINB, GRAD, TJS>;
+  done = false;
+  // per device: the attribute is a property of the function on that device
+  static int occ_dev[VDS_MAX_DEVICES] = {};
+  int &occ = occ_dev[c->device < VDS_MAX_DEVICES ? c->device : 0];
+  if (occ <= 0 || c->device >= VDS_MAX_DEVICES) {
+    VDS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int o = 0;
+    VDS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, NT, smem));
+    occ = o > 0 ? o : 1;
+  }
+  sc.TI = TI;
+  sc.Npad = sc.Nipad = (N + TJ - 1) / TJ * TJ;  // rows of the record array
+  sc.nchunk = (N + TJS - 1) / TJS;
+  sc.cpt = TI / TJS;
+  sc.n_itiles = (N + TI - 1) / TI;
+  sc.items = sched_start(sc.n_itiles, sc);
+  // CTAs per SM: all that fit, or the fewer of them whose largest share of an
+  // SM's items is smaller by more than 3 % (N = 10007, D = 6, 64-thread CTAs:
+  // 41.3 items per SM, which eight CTAs take as 8 x 6 and seven as 7 x 6)
+  auto cost = [&](int o) {
+    const long long g = (long long)c->num_sms * o;
+    return o * ((sc.items + g - 1) / g);
+  };
+  int per = occ;
+  for (int o = occ - 1; 2 * o >= occ; --o)
+    if (100 * cost(o) < 97 * cost(per)) per = o;
+  const long long cap = (long long)c->num_sms * per;
+  sc.G = (int)(sc.items < cap ? sc.items : cap);
+  sc.maxseg = sched_maxseg(sc);
+  const size_t jbytes = (size_t)sched_jrow(sc.n_itiles - 1, sc) * ACC * sizeof(float2);
+  if (jbytes > SYM_MAX_PARTJ) return VDS_OK;
+  int st = vds_ensure(c, c->part, (size_t)sc.n_itiles * sc.maxseg * TI * ACC * sizeof(float2));
+  if (st == VDS_OK && jbytes) st = vds_ensure(c, c->partj, jbytes);
+  if (st == VDS_ENOMEM) {
+    (void)cudaGetLastError();
+    return VDS_OK;
+  }
+  VDS_TRY(st);
+  const int pk = GRAD ? PK_GRADIENT : PK_DENSITY;
+  VDS_TRY(vds_time_begin(c, pk));
+  kern<<<sc.G, NT, smem, c->stream>>>((const float *)c->rec.ptr, sc, N, (float2 *)c->part.ptr,
+                                      (float2 *)c->partj.ptr);
+  VDS_CUDA_TRY(cudaGetLastError());
+  VDS_TRY(vds_time_end(c, pk));
+  ++c->launches;
+  done = true;
+  return VDS_OK;
+}
+
+// The pass of the N particles at c->rec against themselves.
+template <int D, bool GRAD>
+int launch_self(vds_ctx *c, int N, PartSrc &src) {
+  bool done = false;
+  if constexpr (GRAD) {
+    if (N >= SYM_LARGE_N) VDS_TRY((launch_sym<D, true, SymCfg<D, true>::NT_LARGE, 32>(c, N, src.sc, done)));
+    else if (N >= SYM_MIN_N) VDS_TRY((launch_sym<D, true, 128, 32>(c, N, src.sc, done)));
+  } else {
+    if (N >= SYM_CHUNK_N) VDS_TRY((launch_sym<D, false, 128, 64>(c, N, src.sc, done)));
+    else if (N >= SYM_MIN_N) VDS_TRY((launch_sym<D, false, 128, 32>(c, N, src.sc, done)));
+  }
+  if (!done) VDS_TRY((launch_pass<D, GRAD>(c, N, src.sc, N, (const float *)c->rec.ptr)));
+  src.i = (const float2 *)c->part.ptr;
+  src.j = (const float2 *)c->partj.ptr;
+  return VDS_OK;
+}
+
+// Epilogue launches, by the space dimension S of D = nb S.
+template <int D>
+int launch_dens_finish(cudaStream_t st, const PartSrc &src, const KParams &kp, const FinArgs &A) {
+  using F = FinCfg<D>;
+  const int nb = (kp.N + F::PB - 1) / F::PB;
+  if constexpr (D % 2 == 0)
+    if (kp.s == 2) k_dens_finish<D, 2><<<nb, F::NT, 0, st>>>(src, kp, A);
+  if constexpr (D % 3 == 0)
+    if (kp.s == 3) k_dens_finish<D, 3><<<nb, F::NT, 0, st>>>(src, kp, A);
+  VDS_CUDA_TRY(cudaGetLastError());
+  return VDS_OK;
+}
+
+template <int D, int MODE>
+int launch_grad_finish(cudaStream_t st, const PartSrc &src, const KParams &kp, const FinArgs &A) {
+  using F = FinCfg<D>;
+  const int nb = (kp.N + F::PB - 1) / F::PB;
+  if constexpr (D % 2 == 0)
+    if (kp.s == 2) k_grad_finish<D, 2, MODE><<<nb, F::NT, 0, st>>>(src, kp, A);
+  if constexpr (D % 3 == 0)
+    if (kp.s == 3) k_grad_finish<D, 3, MODE><<<nb, F::NT, 0, st>>>(src, kp, A);
+  VDS_CUDA_TRY(cudaGetLastError());
+  return VDS_OK;
+}
+
+// CTAs of an epilogue, each of which leaves up to three FP64 partials.
+template <int D>
+size_t fin_red_bytes(int N) {
+  return (size_t)((N + FinCfg<D>::PB - 1) / FinCfg<D>::PB) * 3 * sizeof(double);
 }
 
 template <int D>
 int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
-                 const float *ybase, const float *ydelta, const float *qa, const float *qb, bool expand) {
-  Sched sc;
-  if (expand)
-    VDS_TRY((launch_pass<D, false, true>(c, kp.N, sc, kp.N, (const float *)c->rec.ptr)));
-  else
-    VDS_TRY((launch_pass<D, false>(c, kp.N, sc, kp.N, (const float *)c->rec.ptr)));
-  const int nb = (kp.N + NT_FIN - 1) / NT_FIN;
-  VDS_TRY(vds_ensure(c, c->red, (size_t)nb * 4 * sizeof(double)));
-  k_dens_finish<D><<<nb, NT_FIN, 0, c->stream>>>(sc, (const double *)c->part.ptr, (float *)c->rec.ptr,
-                                                 rho_out, kp, want_energy ? 1 : 0, ybase, ydelta, qa,
-                                                 qb, (double *)c->red.ptr, c->ticket + TK_DENS,
-                                                 c->scal, c->err);
-  VDS_CUDA_TRY(cudaGetLastError());
+                 const float *ybase, const float *ydelta, const float *qa, const float *qb) {
+  PartSrc src;
+  VDS_TRY((launch_self<D, false>(c, kp.N, src)));
+  VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
+  const FinArgs A{(float *)c->rec.ptr, rho_out, ybase, ydelta, qa, qb, nullptr, want_energy ? 1 : 0,
+                  (double *)c->red.ptr, c->ticket + TK_DENS, c->scal, c->err};
+  VDS_TRY((launch_dens_finish<D>(c->stream, src, kp, A)));
   ++c->launches;
   return VDS_OK;
 }
@@ -736,45 +571,34 @@ int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy
 template <int D>
 int grad_impl(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,
               const float *ydelta, const float *qa, const float *qb, float *q_io) {
-  Sched sc;
-  VDS_TRY((launch_pass<D, true>(c, kp.N, sc, kp.N, (const float *)c->rec.ptr)));
-  const int nb = (kp.N + NT_FIN - 1) / NT_FIN;
-  VDS_TRY(vds_ensure(c, c->red, (size_t)nb * 4 * sizeof(double)));
-  const double *pp = (const double *)c->part.ptr;
-  float *rp = (float *)c->rec.ptr;
-  double *red = (double *)c->red.ptr;
-  unsigned *tk = c->ticket + TK_GRAD;
-  if (mode == GM_OUT)
-    k_grad_finish<D, GM_OUT><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rp, kp, out, ybase, ydelta, qa, qb,
-                                                          q_io, red, tk, c->scal, c->err);
-  else if (mode == GM_EXPLICIT)
-    k_grad_finish<D, GM_EXPLICIT><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rp, kp, out, ybase, ydelta, qa,
-                                                               qb, q_io, red, tk, c->scal, c->err);
-  else if (mode == GM_VEL)
-    k_grad_finish<D, GM_VEL><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rp, kp, out, ybase, ydelta, qa, qb,
-                                                          q_io, red, tk, c->scal, c->err);
-  else
-    k_grad_finish<D, GM_IMPLICIT_DIR><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rp, kp, out, ybase, ydelta,
-                                                                   qa, qb, q_io, red, tk, c->scal,
-                                                                   c->err);
-  VDS_CUDA_TRY(cudaGetLastError());
+  PartSrc src;
+  VDS_TRY((launch_self<D, true>(c, kp.N, src)));
+  VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
+  const FinArgs A{(float *)c->rec.ptr, out, ybase, ydelta, qa, qb, q_io, 0,
+                  (double *)c->red.ptr, c->ticket + TK_GRAD, c->scal, c->err};
+  if (mode == GM_OUT) VDS_TRY((launch_grad_finish<D, GM_OUT>(c->stream, src, kp, A)));
+  else if (mode == GM_EXPLICIT) VDS_TRY((launch_grad_finish<D, GM_EXPLICIT>(c->stream, src, kp, A)));
+  else if (mode == GM_VEL) VDS_TRY((launch_grad_finish<D, GM_VEL>(c->stream, src, kp, A)));
+  else VDS_TRY((launch_grad_finish<D, GM_IMPLICIT_DIR>(c->stream, src, kp, A)));
   ++c->launches;
   return VDS_OK;
 }
 
 // f at the query points: the segment partials of each query summed in a
-// fixed order (FP64), times (1/N)(2 pi h^2)^(-D/2).
+// fixed order, times (1/N)(2 pi h^2)^(-D/2).
+constexpr int NT_FIN = 256;
+
 template <int D>
 __global__ void __launch_bounds__(NT_FIN)
-    k_query_finish(Sched sc, const double *__restrict__ part, int M, double scale, float *__restrict__ f_out,
+    k_query_finish(PartSrc src, int M, double scale, float *__restrict__ f_out,
                    int *err) {
   const int i = blockIdx.x * NT_FIN + threadIdx.x;
   if (i >= M) return;
-  const int t = i / sc.TI, il = i - t * sc.TI;
-  const int f = sched_first_cta((long long)t * sc.nchunk, sc);
-  const int l = sched_first_cta((long long)(t + 1) * sc.nchunk - 1, sc);
-  double s = 0.0;
-  for (int g = 0; g <= l - f; ++g) s += part[((size_t)t * sc.maxseg + g) * sc.TI + il];
+  int nseg;
+  const int n = part_count(src, i, nseg);
+  Sum2 t;
+  for (int x = 0; x < n; ++x) t.add(part_get<1>(src, i, 0, x, nseg));
+  const double s = t.value();
   if (!(s >= 0.0 && s <= 1e300)) vds_flag(err, VDS_ENAN);
   f_out[i] = (float)(s * scale);
 }
@@ -788,9 +612,11 @@ int query_impl(vds_ctx *c, const KParams &kp, const float *q, const float *y, in
                                                        (float *)c->recq.ptr);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
-  Sched sc;
-  VDS_TRY((launch_pass<D, false>(c, kp.N, sc, M, (const float *)c->recq.ptr)));
-  k_query_finish<D><<<(M + NT_FIN - 1) / NT_FIN, NT_FIN, 0, c->stream>>>(sc, (const double *)c->part.ptr, M,
+  PartSrc src;
+  VDS_TRY((launch_pass<D, false>(c, kp.N, src.sc, M, (const float *)c->recq.ptr)));
+  src.i = (const float2 *)c->part.ptr;
+  src.j = nullptr;
+  k_query_finish<D><<<(M + NT_FIN - 1) / NT_FIN, NT_FIN, 0, c->stream>>>(src, M,
                                                                          exp(kp.lnorm), f_out, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
@@ -855,10 +681,11 @@ template <int D>
 int rows_density_impl(vds_ctx *c, const KParams &kp, const float *q, int row0, int nrows, float *rho_rows) {
   VDS_TRY(prep_impl<D>(c, kp, q, nullptr, nullptr, 0.f, nullptr));
   VDS_TRY(rows_records<D>(c, row0, nrows));
-  Sched sc;
-  VDS_TRY((launch_pass<D, false>(c, kp.N, sc, nrows, (const float *)c->recq.ptr)));
-  k_query_finish<D><<<(nrows + NT_FIN - 1) / NT_FIN, NT_FIN, 0, c->stream>>>(sc, (const double *)c->part.ptr,
-                                                                             nrows, 1.0, rho_rows, c->err);
+  PartSrc src;
+  VDS_TRY((launch_pass<D, false>(c, kp.N, src.sc, nrows, (const float *)c->recq.ptr)));
+  src.i = (const float2 *)c->part.ptr;
+  src.j = nullptr;
+  k_query_finish<D><<<(nrows + NT_FIN - 1) / NT_FIN, NT_FIN, 0, c->stream>>>(src, nrows, 1.0, rho_rows, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   return VDS_OK;
@@ -875,21 +702,16 @@ int rows_grad_impl(vds_ctx *c, const KParams &kp, const float *q, const float *r
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   VDS_TRY(rows_records<D>(c, row0, nrows));
-  Sched sc;
-  VDS_TRY((launch_pass<D, true>(c, kp.N, sc, nrows, (const float *)c->recq.ptr)));
+  PartSrc src;
+  VDS_TRY((launch_pass<D, true>(c, kp.N, src.sc, nrows, (const float *)c->recq.ptr)));
+  src.i = (const float2 *)c->part.ptr;
+  src.j = nullptr;
   KParams kl = kp;
   kl.N = nrows;
-  const int nb = (nrows + NT_FIN - 1) / NT_FIN;
-  const double *pp = (const double *)c->part.ptr;
-  float *rq = (float *)c->recq.ptr;
-  const float *y = q + (size_t)row0 * D;
-  if (mode == 0)
-    k_grad_finish<D, GM_OUT><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rq, kl, out, y, nullptr, nullptr, nullptr,
-                                                          nullptr, nullptr, nullptr, c->scal, c->err);
-  else
-    k_grad_finish<D, GM_EXPLICIT><<<nb, NT_FIN, 0, c->stream>>>(sc, pp, rq, kl, nullptr, y, nullptr, nullptr,
-                                                               nullptr, out, nullptr, nullptr, c->scal, c->err);
-  VDS_CUDA_TRY(cudaGetLastError());
+  const FinArgs A{(float *)c->recq.ptr, mode == 0 ? out : nullptr, q + (size_t)row0 * D, nullptr, nullptr, nullptr,
+                  mode == 0 ? nullptr : out, 0, nullptr, nullptr, c->scal, c->err};
+  if (mode == 0) VDS_TRY((launch_grad_finish<D, GM_OUT>(c->stream, src, kl, A)));
+  else VDS_TRY((launch_grad_finish<D, GM_EXPLICIT>(c->stream, src, kl, A)));
   ++c->launches;
   return VDS_OK;
 }
@@ -932,9 +754,8 @@ int flow_impl(vds_ctx *c, const KParams &kp, const float *q, float *qs) {
   }                                                                                           \
   int vds_density_##DD(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,       \
                        const float *ybase, const float *ydelta, const float *qa,              \
-                       const float *qb, bool expand) {                                        \
-    return vds_pair::density_impl<DD>(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb,     \
-                                      expand);                                                \
+                       const float *qb) {                                                     \
+    return vds_pair::density_impl<DD>(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb);    \
   }                                                                                           \
   int vds_grad_##DD(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,  \
                     const float *ydelta, const float *qa, const float *qb, float *q_io) {     \

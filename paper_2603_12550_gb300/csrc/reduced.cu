@@ -469,16 +469,16 @@ struct Dev {
 // The density of every particle of the records in ctx->rec for the passes
 // held to 1e-4 or looser (the refresh's lifted state, the surrogate's
 // subset check): the pair dot products on the tensor cores where the records
-// allow it (D = 6, 9), else the expanded distances on the CUDA cores.  The
+// allow it (D = 6, 9), else the full-order path's density pass.  The
 // tensor-core sums lose more to the |q|^2 terms at single particles (3.4e-4
 // at the worst particle of a cloud stretched five-fold), but X^B, a sum over
-// all particles, stays as close to the oracle as with the FP32 expanded form
+// all particles, stays as close to the oracle as with FP32 expanded distances
 // (N = 65536, r = 10: 3.8e-6 and 1.2e-5 relative at equilibrium and at a
 // three-fold stretch, against 4.5e-6 and 1.5e-5).
 int density_1e4(vds_ctx *c, const KParams &kp, const float *qt) {
   const int st = pass_density_tc(c, kp, nullptr);
   if (st != VDS_EARG) return st;
-  return pass_density(c, kp, nullptr, false, qt, nullptr, nullptr, nullptr, true);
+  return pass_density(c, kp, nullptr, false, qt, nullptr, nullptr, nullptr);
 }
 
 // Lift P, evaluate the density at the lifted state, run the refresh pass and

@@ -209,7 +209,7 @@ void vds_destroy(vds_ctx *c) {
   DeviceGuard g(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
-  DevBuf *bufs[] = {&c->rec, &c->recq, &c->part, &c->red, &c->vecs, &c->gbuf, &c->ubuf, &c->dtbuf};
+  DevBuf *bufs[] = {&c->rec, &c->recq, &c->part, &c->partj, &c->red, &c->vecs, &c->gbuf, &c->ubuf, &c->dtbuf};
   for (DevBuf *b : bufs)
     if (b->ptr) cudaFree(b->ptr);
   if (c->err) cudaFree(c->err);

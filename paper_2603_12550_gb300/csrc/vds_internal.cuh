@@ -192,6 +192,7 @@ struct vds_ctx {
   DevBuf rec;      // records (N_pad x DP floats)
   DevBuf recq;     // records of query points (vds_density_at)
   DevBuf part;     // pair-pass partial sums (FP64)
+  DevBuf partj;    // j-side partial sums of the symmetric passes (FP64)
   DevBuf red;      // block partials of reductions (FP64)
   DevBuf vecs;     // minimiser vectors / scratch (FP32)
   DevBuf gbuf;     // Gram / projection partials (FP64)
