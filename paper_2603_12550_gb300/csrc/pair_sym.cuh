@@ -32,12 +32,6 @@
 
 namespace vds_pair {
 
-// 16-byte asynchronous copy global -> shared of the calling thread.
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // The ACC sums of one j as float4 / float2 / float planes of TJS slots.
 template <int ACC, int TJS>
 struct JSlots {

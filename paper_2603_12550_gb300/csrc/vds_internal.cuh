@@ -122,6 +122,12 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
       : "memory");
 }
 
+// 16-byte asynchronous copy global -> shared of the calling thread.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 #define VDS_WAIT_LIMIT_NS 2000000000ull  // 2 s
 
 // Per-device caches of launch attributes cover devices 0 .. VDS_MAX_DEVICES-1.
