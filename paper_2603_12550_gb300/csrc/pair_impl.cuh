@@ -4,7 +4,7 @@
 //
 // k_pair is the ordered form (rows of any points against all particles): the
 // queries, the row ranges and the allocation-free evaluation; a cloud against
-// itself takes the symmetric form of pair_sym.cuh from SYM_MIN_N particles on.
+// itself takes the symmetric form of pair_sym.cuh from sym_min_n() particles on.
 //
 // Density pass (Eq. model_DeteParAppr, denominators of Eq. model_DymRepPar):
 //   rho_I = sum_J exp2(-|qhat_I - qhat_J|^2),  qhat = c q,  c^2 = log2(e)/(2h^2)
@@ -22,6 +22,7 @@
 
 #include "pair.cuh"
 #include "pair_fin.cuh"
+#include "pair_small.cuh"
 #include "pair_sym.cuh"
 
 namespace vds_pair {
@@ -442,7 +443,11 @@ struct SymCfg {
 // The j sums of a symmetric pass may take this much workspace; larger clouds
 // (and a workspace that cannot be had) take the ordered form.
 constexpr size_t SYM_MAX_PARTJ = (size_t)4 << 30;
-constexpr int SYM_MIN_N = 2048;
+// Smaller clouds take k_small.  Explicit step, k_small / symmetric passes:
+// N = 4096, D = 2 25 / 29 us, D = 9 49 / 63, D = 16 72 / 75; N = 6144, D = 3
+// 45 / 53, D = 6 76 / 81, D = 9 108 / 83.
+template <int D>
+constexpr int sym_min_n() { return D <= 6 ? 6145 : 4865; }
 // From here on the gradient pass takes one CTA per SM: a third of the i-tiles
 // and of the j sums written and read (N = 65536, D = 9: 65 instead of 199 MB).
 constexpr int SYM_LARGE_N = 49152;
@@ -513,10 +518,10 @@ int launch_self(vds_ctx *c, int N, PartSrc &src) {
   bool done = false;
   if constexpr (GRAD) {
     if (N >= SYM_LARGE_N) VDS_TRY((launch_sym<D, true, SymCfg<D, true>::NT_LARGE, 32>(c, N, src.sc, done)));
-    else if (N >= SYM_MIN_N) VDS_TRY((launch_sym<D, true, 128, 32>(c, N, src.sc, done)));
+    else VDS_TRY((launch_sym<D, true, 128, 32>(c, N, src.sc, done)));
   } else {
     if (N >= SYM_CHUNK_N) VDS_TRY((launch_sym<D, false, 128, 64>(c, N, src.sc, done)));
-    else if (N >= SYM_MIN_N) VDS_TRY((launch_sym<D, false, 128, 32>(c, N, src.sc, done)));
+    else VDS_TRY((launch_sym<D, false, 128, 32>(c, N, src.sc, done)));
   }
   if (!done) VDS_TRY((launch_pass<D, GRAD>(c, N, src.sc, N, (const float *)c->rec.ptr)));
   src.i = (const float2 *)c->part.ptr;
@@ -555,14 +560,51 @@ size_t fin_red_bytes(int N) {
   return (size_t)((N + FinCfg<D>::PB - 1) / FinCfg<D>::PB) * 3 * sizeof(double);
 }
 
+// Small clouds: pass and epilogue in one launch.
+template <int D, int MODE, int RI, int NT>
+int launch_small_shape(vds_ctx *c, const KParams &kp, const FinArgs &A) {
+  const int nb = (kp.N + 8 * RI - 1) / (8 * RI);
+  const float *rec = (const float *)c->rec.ptr;
+  VDS_TRY(vds_ensure(c, c->red, (size_t)nb * 3 * sizeof(double)));
+  FinArgs B = A;
+  B.red = (double *)c->red.ptr;
+  const int pk = MODE == SM_DENS ? PK_DENSITY : PK_GRADIENT;
+  VDS_TRY(vds_time_begin(c, pk));
+  if constexpr (D % 2 == 0)
+    if (kp.s == 2) k_small<D, 2, RI, NT, MODE><<<nb, NT, 0, c->stream>>>(rec, kp, B);
+  if constexpr (D % 3 == 0)
+    if (kp.s == 3) k_small<D, 3, RI, NT, MODE><<<nb, NT, 0, c->stream>>>(rec, kp, B);
+  VDS_CUDA_TRY(cudaGetLastError());
+  VDS_TRY(vds_time_end(c, pk));
+  ++c->launches;
+  return VDS_OK;
+}
+
+// Particles per lane: one while that leaves at most two CTAs per SM; two or,
+// where the registers of D = 8 to 10 make the most of it, four above (N = 4096:
+// D = 3 34 / 33 / 31 us a step with 1 / 2 / 4, D = 6 57 / 36 / 41, D = 9
+// 70 / 58 / 49, D = 16 136 / 72 / 108).
+// 1024 threads per CTA where an SM has one CTA (or D leaves the registers for
+// two), 512 otherwise: N = 1000, D = 9 11.7 / 14.3 / 19.0 us with 1024 / 512 /
+// 256; N = 1536, D = 9 19.7 / 18.8.
+template <int D, int MODE>
+int launch_small(vds_ctx *c, const KParams &kp, const FinArgs &A) {
+  constexpr int RI1_N = D <= 10 ? 2432 : 1216, RI2 = D >= 8 && D <= 10 ? 4 : 2;
+  if (kp.N > RI1_N) return launch_small_shape<D, MODE, RI2, (8 * RI2 * D > 512 ? 1024 : 512)>(c, kp, A);
+  if (D <= 3 || kp.N <= 8 * c->num_sms) return launch_small_shape<D, MODE, 1, 1024>(c, kp, A);
+  return launch_small_shape<D, MODE, 1, 512>(c, kp, A);
+}
+
 template <int D>
 int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
                  const float *ybase, const float *ydelta, const float *qa, const float *qb) {
+  FinArgs A{(float *)c->rec.ptr, rho_out, ybase, ydelta, qa, qb, nullptr, want_energy ? 1 : 0,
+            nullptr, c->ticket + TK_DENS, c->scal, c->err};
+  if (kp.N < sym_min_n<D>()) return launch_small<D, SM_DENS>(c, kp, A);
   PartSrc src;
   VDS_TRY((launch_self<D, false>(c, kp.N, src)));
   VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
-  const FinArgs A{(float *)c->rec.ptr, rho_out, ybase, ydelta, qa, qb, nullptr, want_energy ? 1 : 0,
-                  (double *)c->red.ptr, c->ticket + TK_DENS, c->scal, c->err};
+  A.red = (double *)c->red.ptr;
   VDS_TRY((launch_dens_finish<D>(c->stream, src, kp, A)));
   ++c->launches;
   return VDS_OK;
@@ -571,11 +613,25 @@ int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy
 template <int D>
 int grad_impl(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,
               const float *ydelta, const float *qa, const float *qb, float *q_io) {
+  FinArgs A{(float *)c->rec.ptr, out, ybase, ydelta, qa, qb, q_io, 0, nullptr, c->ticket + TK_GRAD, c->scal, c->err};
+  if (kp.N < sym_min_n<D>()) {
+    if (mode == GM_OUT) return launch_small<D, GM_OUT>(c, kp, A);
+    if (mode == GM_VEL) return launch_small<D, GM_VEL>(c, kp, A);
+    if (mode == GM_IMPLICIT_DIR) return launch_small<D, GM_IMPLICIT_DIR>(c, kp, A);
+    // the records of the next step go to the other array: CTAs that are still
+    // summing read this one
+    VDS_TRY(vds_ensure(c, c->rec2, (size_t)pass_npad(kp.N) * Rec<D>::DP * sizeof(float)));
+    A.rec = (float *)c->rec2.ptr;
+    VDS_TRY((launch_small<D, GM_EXPLICIT>(c, kp, A)));
+    const DevBuf t = c->rec;
+    c->rec = c->rec2;
+    c->rec2 = t;
+    return VDS_OK;
+  }
   PartSrc src;
   VDS_TRY((launch_self<D, true>(c, kp.N, src)));
   VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
-  const FinArgs A{(float *)c->rec.ptr, out, ybase, ydelta, qa, qb, q_io, 0,
-                  (double *)c->red.ptr, c->ticket + TK_GRAD, c->scal, c->err};
+  A.red = (double *)c->red.ptr;
   if (mode == GM_OUT) VDS_TRY((launch_grad_finish<D, GM_OUT>(c->stream, src, kp, A)));
   else if (mode == GM_EXPLICIT) VDS_TRY((launch_grad_finish<D, GM_EXPLICIT>(c->stream, src, kp, A)));
   else if (mode == GM_VEL) VDS_TRY((launch_grad_finish<D, GM_VEL>(c->stream, src, kp, A)));

@@ -209,7 +209,7 @@ void vds_destroy(vds_ctx *c) {
   DeviceGuard g(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
-  DevBuf *bufs[] = {&c->rec, &c->recq, &c->part, &c->partj, &c->red, &c->vecs, &c->gbuf, &c->ubuf, &c->dtbuf};
+  DevBuf *bufs[] = {&c->rec, &c->rec2, &c->recq, &c->part, &c->partj, &c->red, &c->vecs, &c->gbuf, &c->ubuf, &c->dtbuf};
   for (DevBuf *b : bufs)
     if (b->ptr) cudaFree(b->ptr);
   if (c->err) cudaFree(c->err);
@@ -323,11 +323,12 @@ int vds_density_at(vds_ctx *c, const float *q, int N, int D, const vds_params *p
 }
 
 // Explicit steps.  After the first (launched directly; it sizes every buffer
-// a step uses), the steps replay one captured CUDA graph of a step (density
-// pass, its epilogue, gradient pass, the fused update: four kernels with the
-// same arguments every step), which takes the per-launch host cost out of
-// small clouds.  With phase timing on (its events belong to single
-// launches), or if the capture fails, the steps are launched one by one.
+// a step uses), pairs of steps replay one captured CUDA graph (density pass,
+// its epilogue, gradient pass, the fused update; two steps, after which the
+// record arrays that small clouds alternate between are where they were),
+// which takes the per-launch host cost out of small clouds.  With phase
+// timing on (its events belong to single launches), or if the capture fails,
+// the steps are launched one by one, as is an odd last one.
 static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
   VDS_TRY(pass_prep(c, kp, q, nullptr, nullptr, 0.f, nullptr));
   auto one_step = [&]() -> int {
@@ -340,11 +341,12 @@ static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
     ++n;
   }
   cudaGraphExec_t gexec = nullptr;
-  long per_step = 0;
-  if (nsteps - n >= 2 && !(c->timing && c->timing->on)) {
+  long per_replay = 0;
+  if (nsteps - n >= 4 && !(c->timing && c->timing->on)) {
     // captured on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured), launched on the caller's stream
     const long l0 = c->launches;
+    const DevBuf rec = c->rec, rec2 = c->rec2;
     cudaGraph_t g = nullptr;
     cudaStream_t cs = nullptr, user = c->stream;
     int st = VDS_OK;
@@ -355,6 +357,7 @@ static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
     } else {
       c->stream = cs;
       st = one_step();
+      if (st == VDS_OK) st = one_step();
       c->stream = user;
       const cudaError_t ec = cudaStreamEndCapture(cs, &g);
       if (st == VDS_OK && ec != cudaSuccess) st = VDS_ECUDA;
@@ -366,21 +369,23 @@ static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
       st = VDS_ECUDA;
     }
     if (g) cudaGraphDestroy(g);
-    per_step = c->launches - l0;
+    per_replay = c->launches - l0;
     c->launches = l0;
     if (st != VDS_OK) {
       (void)cudaGetLastError();  // a failed capture leaves its status behind
+      c->rec = rec;  // and may have ended between the two steps
+      c->rec2 = rec2;
       if (gexec) cudaGraphExecDestroy(gexec);
       gexec = nullptr;
     }
   }
   int st = VDS_OK;
-  for (; n < nsteps && gexec; ++n) {
+  for (; n + 2 <= nsteps && gexec; n += 2) {
     if (cudaGraphLaunch(gexec, c->stream) != cudaSuccess) {
       st = VDS_ECUDA;
       break;
     }
-    c->launches += per_step;
+    c->launches += per_replay;
   }
   for (; st == VDS_OK && n < nsteps; ++n) st = one_step();
   const int sst = vds_sync_status(c);  // the replays have finished before the graph goes

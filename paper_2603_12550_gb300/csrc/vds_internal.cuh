@@ -196,6 +196,7 @@ struct vds_ctx {
   cudaStream_t stream = nullptr;
   // workspace, grown on demand
   DevBuf rec;      // records (N_pad x DP floats)
+  DevBuf rec2;     // the next step's records while a small cloud's pass reads rec
   DevBuf recq;     // records of query points (vds_density_at)
   DevBuf part;     // pair-pass partial sums (FP64)
   DevBuf partj;    // j-side partial sums of the symmetric passes (FP64)
