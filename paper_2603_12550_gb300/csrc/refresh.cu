@@ -191,26 +191,12 @@ __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsig
   return r;
 }
 
-// One probe of an mbarrier phase that may suspend the thread (up to 20 us)
-// until the phase completes, so that waiting roles do not take issue slots
-// from the warps sharing their scheduler.
-__device__ __forceinline__ bool rc_try_wait_sleep(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(20000u)
-      : "memory");
-  return ok != 0;
-}
 // Wait that also gives up as soon as another role has aborted.
 __device__ __forceinline__ bool rc_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
   for (;;) {
-    if (rc_try_wait_sleep(bar, parity)) return true;
+    if (mbar_try_wait_sleep(bar, parity)) return true;
     if (*abort) return false;
     if (global_timer_ns() - t0 > VDS_WAIT_LIMIT_NS) {
       *abort = 1;
