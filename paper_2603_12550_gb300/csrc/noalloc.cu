@@ -164,11 +164,11 @@ int na_energy_grad(const DevState &s, const float *q, const KParams &kp, double 
   src.i = part;
   src.j = nullptr;
   VDS_TRY((na_pair<D, false>(s, N, st, rec, part, err, src.sc)));
-  const FinArgs ad{rec, rho, q, nullptr, nullptr, nullptr, nullptr, E ? 1 : 0, red, ticket + TK_DENS, scal, err};
+  const FinArgs ad{rec, rho, q, nullptr, nullptr, nullptr, nullptr, E ? 1 : 0, red, ticket + TK_DENS, scal, err, ImpArgs{}};
   VDS_TRY((launch_dens_finish<D>(st, src, kp, ad)));
   if (g) {
     VDS_TRY((na_pair<D, true>(s, N, st, rec, part, err, src.sc)));
-    const FinArgs ag{rec, g, q, nullptr, nullptr, nullptr, nullptr, 0, red, ticket + TK_GRAD, scal, err};
+    const FinArgs ag{rec, g, q, nullptr, nullptr, nullptr, nullptr, 0, red, ticket + TK_GRAD, scal, err, ImpArgs{}};
     VDS_TRY((launch_grad_finish<D, GM_OUT>(st, src, kp, ag)));
   }
   double e_host = 0.0;

@@ -7,10 +7,31 @@
 #include "pair_impl.cuh"
 
 namespace {
-__global__ void k_axpy(int n, const float *__restrict__ a, const float *__restrict__ b,
-                       float *__restrict__ o) {
+// End of an implicit step: q = q* + d, d = d[cur] (- dir) kept for the next
+// step's start; the last CTA closes the step.
+__global__ void __launch_bounds__(256)
+    k_imp_end(int n, ImpArgs imp, const float *__restrict__ qs, const float *__restrict__ dir, float *__restrict__ q,
+              int *__restrict__ iters, unsigned *ticket) {
+  ImpState *s = imp.st;
+  if (s->phase != IMP_FINAL) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) o[i] = a[i] + b[i];
+  if (i < n) {
+    const float *dcur = s->cur ? imp.d[1] : imp.d[0];
+    float *doth = s->cur ? imp.d[0] : imp.d[1];
+    float d = dcur[i];
+    if (s->fin_dir) d = d - 1.f * dir[i];
+    doth[i] = d;
+    q[i] = qs[i] + d;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(ticket, 1u) != gridDim.x - 1) return;
+  *ticket = 0u;
+  iters[s->step] = s->it;
+  s->cur = 1 - s->cur;
+  ++s->step;
+  s->phase = s->status ? IMP_STOP : IMP_READY;
 }
 
 }  // namespace
@@ -33,70 +54,81 @@ __global__ void k_axpy(int n, const float *__restrict__ a, const float *__restri
   }
 
 int vds_prep_2(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_2(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_2(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_2(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_2(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_2(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_2(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_2(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_2(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_2(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_3(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_3(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_3(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_3(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_3(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_3(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_3(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_3(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_3(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_3(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_4(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_4(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_4(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_4(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_4(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_4(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_4(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_4(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_4(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_4(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_6(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_6(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_6(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_6(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_6(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_6(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_6(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_6(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_6(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_6(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_8(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_8(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_8(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_8(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_8(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_8(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_8(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_8(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_8(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_8(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_9(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_9(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_9(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_9(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_9(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_9(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_9(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_9(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_9(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_9(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_10(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_10(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_10(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_10(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_10(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_10(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_10(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_10(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_10(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_10(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_12(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_12(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_12(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_12(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_12(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_12(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_12(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_12(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_12(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_12(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_14(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_14(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_14(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_14(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_14(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_14(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_14(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_14(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_14(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_14(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_15(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_15(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_15(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_15(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_15(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_15(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_15(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_15(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_15(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_15(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 int vds_prep_16(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
-int vds_density_16(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *);
-int vds_grad_16(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *);
+int vds_density_16(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
+int vds_grad_16(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_16(vds_ctx *, const KParams &, const float *, double *, double *);
-int vds_flow_16(vds_ctx *, const KParams &, const float *, float *);
+int vds_impbegin_16(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
+int vds_imptrial_16(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_16(vds_ctx *, const KParams &, const float *, const float *, int, float *);
 
 int vds_rowsdens_2(vds_ctx *, const KParams &, const float *, int, int, float *);
@@ -139,6 +171,9 @@ KParams make_kparams(const vds_params *p, int N, int D) {
   const double c = sqrt(1.4426950408889634 / (2.0 * p->h * p->h));  // log2(e)/(2h^2)
   k.c = (float)c;
   k.sfac = 1.0 / (p->h * p->h * (double)k.c);
+  k.rzeta = 1.0 / p->zeta;
+  k.zeta_dt = p->dt != 0.0 ? p->zeta / p->dt : 0.0;
+  k.dt_zeta = p->dt / p->zeta;
   k.lnorm = -log((double)N) - 0.5 * D * log(2.0 * 3.14159265358979323846 * p->h * p->h);
   return k;
 }
@@ -153,15 +188,16 @@ int pass_prep(vds_ctx *c, const KParams &kp, const float *base, const float *del
 }
 
 int pass_density(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
-                 const float *ybase, const float *ydelta, const float *qa, const float *qb) {
-#define CALL(DD) vds_density_##DD(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb)
+                 const float *ybase, const float *ydelta, const float *qa, const float *qb,
+                 const ImpArgs *imp) {
+#define CALL(DD) vds_density_##DD(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb, imp)
   VDS_DISPATCH_D(kp.D, CALL)
 #undef CALL
 }
 
 int pass_grad(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,
-              const float *ydelta, const float *qa, const float *qb, float *q_io) {
-#define CALL(DD) vds_grad_##DD(c, kp, mode, out, ybase, ydelta, qa, qb, q_io)
+              const float *ydelta, const float *qa, const float *qb, float *q_io, const ImpArgs *imp) {
+#define CALL(DD) vds_grad_##DD(c, kp, mode, out, ybase, ydelta, qa, qb, q_io, imp)
   VDS_DISPATCH_D(kp.D, CALL)
 #undef CALL
 }
@@ -172,10 +208,25 @@ int pass_stress(vds_ctx *c, const KParams &kp, const float *q, double *tau, doub
 #undef CALL
 }
 
-int pass_flow(vds_ctx *c, const KParams &kp, const float *q, float *qs) {
-#define CALL(DD) vds_flow_##DD(c, kp, q, qs)
+int imp_begin(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *q, float *qs) {
+#define CALL(DD) vds_impbegin_##DD(c, kp, imp, q, qs)
   VDS_DISPATCH_D(kp.D, CALL)
 #undef CALL
+}
+
+int imp_trial(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs, const float *dir) {
+#define CALL(DD) vds_imptrial_##DD(c, kp, imp, qs, dir)
+  VDS_DISPATCH_D(kp.D, CALL)
+#undef CALL
+}
+
+int imp_end(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs, const float *dir, float *q,
+            int *iters) {
+  const int n = kp.N * kp.D;
+  k_imp_end<<<(n + 255) / 256, 256, 0, c->stream>>>(n, imp, qs, dir, q, iters, c->ticket + TK_MISC);
+  VDS_CUDA_TRY(cudaGetLastError());
+  ++c->launches;
+  return VDS_OK;
 }
 
 int pass_density_at(vds_ctx *c, const KParams &kp, const float *q, const float *y, int M, float *f_out) {
@@ -195,11 +246,4 @@ int pass_grad_rows(vds_ctx *c, const KParams &kp, const float *q, const float *r
 #define CALL(DD) vds_rowsgrad_##DD(c, kp, q, rho, row0, nrows, mode, out)
   VDS_DISPATCH_D(kp.D, CALL)
 #undef CALL
-}
-
-int pass_axpy(vds_ctx *c, int n, const float *base, const float *delta, float *out) {
-  k_axpy<<<(n + 255) / 256, 256, 0, c->stream>>>(n, base, delta, out);
-  VDS_CUDA_TRY(cudaGetLastError());
-  ++c->launches;
-  return VDS_OK;
 }

@@ -44,6 +44,35 @@ __host__ __device__ __forceinline__ long long sched_jrow(int t, const Sched &s) 
   return ((long long)t * s.nchunk - (long long)s.cpt * ((long long)t * (t + 1) / 2)) * (s.TI / s.cpt);
 }
 
+// The implicit step's minimiser as the device runs it (vds_capi.cu): which
+// evaluation comes next, and the line search's state.  Kernels launched for an
+// evaluation that is not due return at once.
+enum ImpPhase {
+  IMP_READY = 0,  // between steps (begun by k_imp_begin while step < nsteps)
+  IMP_TRIAL = 1,  // density at the trial point
+  IMP_GRAD = 2,   // gradient and direction at the accepted point
+  IMP_FINAL = 3,  // the step's update of q
+  IMP_STOP = 4    // failed
+};
+struct ImpState {
+  double J, alpha, dec;
+  double tol, jfloor;
+  int phase, it, ls, cur, fin_dir, status;
+  int start;   // the trial is the step's first point
+  int cold;    // ... without the previous step's correction
+  int step, nsteps, max_iter, pad;
+};
+__device__ __forceinline__ bool imp_due(const ImpState *s, bool grad) {
+  const int ph = s->phase;
+  return grad ? ph == IMP_GRAD : (ph == IMP_TRIAL || (ph == IMP_READY && s->step < s->nsteps));
+}
+// What a minimiser's passes take: its state and the two displacement buffers
+// (the accepted one is d[cur], the trial's d[1 - cur]).
+struct ImpArgs {
+  ImpState *st = nullptr;
+  float *d[2] = {nullptr, nullptr};
+};
+
 // Physical parameters as the kernels see them.
 struct KParams {
   int N, D, nb, s, spring;
@@ -53,6 +82,8 @@ struct KParams {
   double kappa[9];
   double lnorm;     // -ln N - (D/2) ln(2 pi h^2)
   double sfac;      // S = -sfac * sum u dqhat, sfac = 1/(h^2 c)
+  // ratios the epilogues use, so that no FP64 division is on their chain
+  double rzeta, zeta_dt, dt_zeta;  // 1/zeta, zeta/dt and dt/zeta (0 where dt = 0)
 };
 
 KParams make_kparams(const vds_params *p, int N, int D);
@@ -72,9 +103,12 @@ int pass_prep(vds_ctx *c, const KParams &kp, const float *base, const float *del
 //   (1/N) sum_I [kBT (ln rho_I + lnorm) + Psi(y_I)]
 //   + (zeta/2dt)(1/N) sum_I dI^T (A^-1 (x) I) dI,   dI = qa_I - qb_I
 // (the quadratic term only when qa != NULL; qb may be NULL) into scal[SC_E].
-// y_I = ybase_I + ydelta_I (ydelta may be NULL).
+// y_I = ybase_I + ydelta_I (ydelta may be NULL).  imp (pass_grad too): the
+// pass of a device-run minimiser, with its displacements in place of ydelta
+// and qa, and its next state set by the epilogue.
 int pass_density(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
-                 const float *ybase, const float *ydelta, const float *qa, const float *qb);
+                 const float *ybase, const float *ydelta, const float *qa, const float *qb,
+                 const ImpArgs *imp = nullptr);
 
 // The same density without the energy, with the pair dot products on the
 // tensor cores (dens_tc.cu: 3xTF32; 1e-5 relative for the median particle of
@@ -99,7 +133,7 @@ enum GradMode { GM_OUT = 0, GM_EXPLICIT = 1, GM_IMPLICIT_DIR = 2, GM_VEL = 3 };
 //   scal[SC_DMAX] = max|dir|, scal[SC_YMAX] = max|y|.
 int pass_grad(vds_ctx *c, const KParams &kp, int mode, float *out,
               const float *ybase, const float *ydelta, const float *qa,
-              const float *qb, float *q_io);
+              const float *qb, float *q_io, const ImpArgs *imp = nullptr);
 
 // Stress and second moments (FP64) into host arrays.
 int pass_stress(vds_ctx *c, const KParams &kp, const float *q, double *tau, double *qq);
@@ -109,10 +143,16 @@ int pass_stress(vds_ctx *c, const KParams &kp, const float *q, double *tau, doub
 // the particles' records built from q, the queries' in their own buffer.
 int pass_density_at(vds_ctx *c, const KParams &kp, const float *q, const float *y, int M, float *f_out);
 
-// y = base + delta -> out (element-wise, N x D).
-int pass_axpy(vds_ctx *c, int n, const float *base, const float *delta, float *out);
-// qs = q + dt kappa q (per bond).
-int pass_flow(vds_ctx *c, const KParams &kp, const float *q, float *qs);
+// The minimiser's own kernels (an implicit step is begin, then passes and
+// trial points by turns, then end; each returns at once where it is not due):
+// imp_begin: q* = q + dt kappa q into qs, the start displacement into the
+//   trial buffer, its records;
+// imp_trial: trial displacement d[cur] - alpha dir, its records;
+// imp_end: q = q* + d[cur] (- dir), which also becomes the next start.
+int imp_begin(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *q, float *qs);
+int imp_trial(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs, const float *dir);
+int imp_end(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs, const float *dir, float *q,
+            int *iters);
 
 // Row-range passes (rows row0 .. row0 + nrows - 1 against all N columns):
 // rho of the rows; and, given rho of all N particles, g of the rows (mode 0)

@@ -44,38 +44,41 @@ struct Sum2 {
 };
 
 // Deterministic grid reduction of K values per thread: warp, CTA, then the
-// last CTA to arrive (ticket) sums the CTAs' partials in a fixed order.
+// last CTA to arrive (ticket) sums the CTAs' partials in a fixed order.  Only
+// the first NA threads of a CTA have values, and only warps that hold some
+// take part: FP64 sums of 32 warps of zeros took 4 us of a pass at N = 512.
 // Returns true in the thread that holds the final value.
-template <int K, int NT>
-__device__ __forceinline__ bool grid_reduce(double (&v)[K], const bool (&is_max)[K], double *red,
+template <int K, int NT, int NA>
+__device__ __forceinline__ bool grid_reduce(const double (&v)[K], const bool (&is_max)[K], double *red,
                                             unsigned *ticket, double (&out)[K]) {
   constexpr int NW = NT / 32;
   __shared__ double sh[NW][K];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  auto cta = [&](double (&x)[K]) {  // result in thread 0
+  auto cta = [&](double (&x)[K], int nw) {  // of the first nw warps; result in thread 0
+    if (w < nw)
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
+      for (int k = 0; k < K; ++k) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double y = __shfl_xor_sync(0xffffffffu, x[k], o);
-        x[k] = is_max[k] ? fmax(x[k], y) : x[k] + y;
+        for (int o = 16; o > 0; o >>= 1) {
+          const double y = __shfl_xor_sync(0xffffffffu, x[k], o);
+          x[k] = is_max[k] ? fmax(x[k], y) : x[k] + y;
+        }
+        if (lane == 0) sh[w][k] = x[k];
       }
-      if (lane == 0) sh[w][k] = x[k];
-    }
     __syncthreads();
     if (threadIdx.x == 0)
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         double s = sh[0][k];
-        for (int q = 1; q < NW; ++q) s = is_max[k] ? fmax(s, sh[q][k]) : s + sh[q][k];
+        for (int q = 1; q < nw; ++q) s = is_max[k] ? fmax(s, sh[q][k]) : s + sh[q][k];
         x[k] = s;
       }
   };
   double x[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) x[k] = v[k];
-  cta(x);
+  cta(x, (NA + 31) / 32);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) red[(size_t)blockIdx.x * K + k] = x[k];
@@ -93,7 +96,8 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[K], const bool (&is_max)
       const double y = __ldcg(red + (size_t)b * K + k);
       x[k] = is_max[k] ? fmax(x[k], y) : x[k] + y;
     }
-  cta(x);
+  const int nw = (int)((gridDim.x + 31u) / 32u);
+  cta(x, nw < NW ? nw : NW);
   if (threadIdx.x != 0) return false;
 #pragma unroll
   for (int k = 0; k < K; ++k) out[k] = x[k];
@@ -165,29 +169,112 @@ struct FinArgs {
   unsigned *ticket;
   double *scal;
   int *err;
+  ImpArgs imp;  // imp.st NULL: not a minimiser's pass
 };
+
+// The displacements of a pass (a copy of the arguments with the minimiser's in
+// their place would put them all in local memory).
+struct FinPtrs {
+  const float *ydelta, *qa;
+};
+// Whether the pass is due (a minimiser's may not be), and its displacements.
+__device__ __forceinline__ bool imp_take(const FinArgs &A, bool grad, FinPtrs &P) {
+  P.ydelta = A.ydelta;
+  P.qa = A.qa;
+  const ImpState *s = A.imp.st;
+  if (!s) return true;
+  if (!imp_due(s, grad)) return false;
+  P.ydelta = (s->cur != 0) == grad ? A.imp.d[1] : A.imp.d[0];
+  if (!grad) P.qa = P.ydelta;
+  return true;
+}
+
+// The minimiser's next state after the trial's objective J.  One thread, after
+// every CTA has raised its flags.
+__device__ __forceinline__ void imp_after_trial(ImpState *s, double J, int *err) {
+  const int e = *(volatile int *)err;
+  const bool start = s->phase == IMP_READY || s->start;
+  if (s->phase == IMP_READY) {
+    s->it = 0;
+    s->cold = s->step == 0;
+  }
+  if (e != 0 && e != VDS_EDOMAIN) {
+    s->phase = IMP_STOP;
+    return;
+  }
+  if (start) {
+    if (e == VDS_EDOMAIN) {
+      if (s->cold) {
+        s->phase = IMP_STOP;  // q* itself is outside
+        return;
+      }
+      *err = 0;
+      s->cold = 1;  // the previous correction leads outside: start from q*
+      s->start = 1;
+      s->alpha = 0.0;
+      s->phase = IMP_TRIAL;
+      return;
+    }
+    s->start = 0;
+  } else if (e == VDS_EDOMAIN || !(J <= s->J - 1e-4 * s->alpha * s->dec + s->jfloor * (1.0 + fabs(s->J)))) {
+    *err = 0;
+    s->alpha *= 0.5;
+    if (++s->ls > 30) {
+      s->status = VDS_ENOCONV;
+      s->phase = IMP_STOP;
+    }
+    return;
+  }
+  s->J = J;
+  s->cur = 1 - s->cur;
+  if (s->it >= s->max_iter) {
+    s->status = VDS_ENOCONV;
+    s->fin_dir = 0;
+    s->phase = IMP_FINAL;
+  } else {
+    s->phase = IMP_GRAD;
+  }
+}
+
+// ... after a direction: decrease dec, largest entries of the direction and of y.
+__device__ __forceinline__ void imp_after_grad(ImpState *s, double dec, double dmax, double ymax, int *err) {
+  if (*(volatile int *)err != 0) {
+    s->phase = IMP_STOP;
+    return;
+  }
+  ++s->it;
+  s->dec = dec;
+  if (dmax <= s->tol * (1.0 + ymax)) {
+    s->fin_dir = 1;
+    s->phase = IMP_FINAL;
+  } else {
+    s->alpha = 1.0;
+    s->ls = 0;
+    s->phase = IMP_TRIAL;
+  }
+}
 
 // y of every particle of the CTA into sh.y (FP32 sum of base and delta), and
 // qa - qb (or ydelta) into sh.d where asked; ends with a barrier.
 template <int D, int PB>
-__device__ __forceinline__ void fin_load(const FinArgs &A, int base, int N, bool want_d, bool d_is_delta,
+__device__ __forceinline__ void fin_load(const FinArgs &A, const FinPtrs &P, int base, int N, bool want_d, bool d_is_delta,
                                          FinShared<D, PB> &sh) {
   const int n = min(PB, N - base) * D;
   const int e = threadIdx.x;
   if (e < n) {
     const size_t x = (size_t)base * D + e;
     float v = A.ybase[x];
-    if (A.ydelta) v = v + A.ydelta[x];
+    if (P.ydelta) v = v + P.ydelta[x];
     sh.y[e % D][e / D] = (double)v;
     if (want_d)
-      sh.d[e % D][e / D] = d_is_delta ? (double)A.ydelta[x] : (double)A.qa[x] - (A.qb ? (double)A.qb[x] : 0.0);
+      sh.d[e % D][e / D] = d_is_delta ? (double)P.ydelta[x] : (double)P.qa[x] - (A.qb ? (double)A.qb[x] : 0.0);
   }
   __syncthreads();
 }
 
 // Density: rho of the particle in every one of its threads.
 template <int D, int S, int PB, int NT>
-__device__ __forceinline__ void fin_density(const KParams &kp, const FinArgs &A, int base, double rho,
+__device__ __forceinline__ void fin_density(const KParams &kp, const FinArgs &A, const FinPtrs &P, int base, double rho,
                                             FinShared<D, PB> &sh) {
   constexpr int DP = Rec<D>::DP, NB = D / S;
   const int p = threadIdx.x % PB, a = threadIdx.x / PB, i = base + p;
@@ -198,7 +285,7 @@ __device__ __forceinline__ void fin_density(const KParams &kp, const FinArgs &A,
     if (A.out) A.out[i] = (float)rho;
   }
   if (!A.want_energy) return;
-  fin_load<D, PB>(A, base, kp.N, A.qa != nullptr, false, sh);
+  fin_load<D, PB>(A, P, base, kp.N, P.qa != nullptr, false, sh);
   double e = 0.0;
   if (on) {
     const int k = a / S, al = a - k * S;
@@ -210,31 +297,33 @@ __device__ __forceinline__ void fin_density(const KParams &kp, const FinArgs &A,
       e += psi;
     }
     if (a == 0) e += kp.kBT * (log(rho) + kp.lnorm);
-    if (A.qa) {
+    if (P.qa) {
       double m = 0.0;
 #pragma unroll
       for (int kb = 0; kb < NB; ++kb) m += rouse_Ainv<NB>(k, kb) * sh.d[kb * S + al][p];
-      e += kp.zeta / (2.0 * kp.dt) * sh.d[a][p] * m;
+      e += 0.5 * kp.zeta_dt * sh.d[a][p] * m;
     }
   }
   double v[1] = {e}, out[1];
   const bool mx[1] = {false};
-  if (grid_reduce<1, NT>(v, mx, A.red, A.ticket, out)) {
-    A.scal[SC_E] = out[0] / (double)kp.N;
-    if (!(fabs(A.scal[SC_E]) <= 1e300)) vds_flag(A.err, VDS_ENAN);
+  if (grid_reduce<1, NT, PB * D>(v, mx, A.red, A.ticket, out)) {
+    const double E = out[0] / (double)kp.N;
+    A.scal[SC_E] = E;
+    if (!(fabs(E) <= 1e300)) vds_flag(A.err, VDS_ENAN);
+    if (A.imp.st) imp_after_trial(A.imp.st, E, A.err);
   }
 }
 
 // Gradient: u_sum is sum_J u dqhat of (particle p, component a).
 template <int D, int S, int MODE, int PB, int NT>
-__device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, int base, double u_sum,
+__device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, const FinPtrs &P, int base, double u_sum,
                                          FinShared<D, PB> &sh) {
   constexpr int DP = Rec<D>::DP, NB = D / S;
   const int p = threadIdx.x % PB, a = threadIdx.x / PB, i = base + p;
   const bool on = i < kp.N && a < D;
   const int k = a / S, al = a - k * S;
-  const bool want_d = MODE == GM_IMPLICIT_DIR || (MODE == GM_OUT && A.qa != nullptr);
-  fin_load<D, PB>(A, base, kp.N, want_d, MODE == GM_IMPLICIT_DIR, sh);
+  const bool want_d = MODE == GM_IMPLICIT_DIR || (MODE == GM_OUT && P.qa != nullptr);
+  fin_load<D, PB>(A, P, base, kp.N, want_d, MODE == GM_IMPLICIT_DIR, sh);
   double g = 0.0;
   if (on) {
     double f = kp.H[k];
@@ -255,7 +344,7 @@ __device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, in
       double m = 0.0;
 #pragma unroll
       for (int kb = 0; kb < NB; ++kb) m += rouse_Ainv<NB>(k, kb) * sh.d[kb * S + al][p];
-      g += kp.zeta / kp.dt * m;
+      g += kp.zeta_dt * m;
     }
   }
   float row = (float)g;  // what this thread contributes to its particle's row
@@ -272,8 +361,8 @@ __device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, in
         double aid = 0.0;
 #pragma unroll
         for (int kb = 0; kb < NB; ++kb) aid += rouse_Ainv<NB>(k, kb) * sh.d[kb * S + al][p];
-        const double dr = sh.d[a][p] + kp.dt / kp.zeta * m;
-        const double G = kp.zeta / kp.dt * aid + g;
+        const double dr = sh.d[a][p] + kp.dt_zeta * m;
+        const double G = kp.zeta_dt * aid + g;
         row = (float)dr;
         dec = G * dr;
         dmax = fabs((double)row);
@@ -282,7 +371,7 @@ __device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, in
         double v = 0.0;
 #pragma unroll
         for (int be = 0; be < S; ++be) v += kp.kappa[al * S + be] * sh.y[k * S + be][p];
-        const double vel = v - m / kp.zeta;
+        const double vel = v - m * kp.rzeta;
         row = MODE == GM_VEL ? (float)vel : (float)(sh.y[a][p] + kp.dt * vel);
       }
     }
@@ -307,17 +396,20 @@ __device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, in
   if constexpr (MODE == GM_IMPLICIT_DIR) {
     double v[3] = {dec, dmax, ymax}, o[3];
     const bool mx[3] = {false, true, true};
-    if (grid_reduce<3, NT>(v, mx, A.red, A.ticket, o)) {
+    if (grid_reduce<3, NT, PB * D>(v, mx, A.red, A.ticket, o)) {
       A.scal[SC_DEC] = o[0] / (double)kp.N;
       A.scal[SC_DMAX] = o[1];
       A.scal[SC_YMAX] = o[2];
       if (!(fabs(o[0]) <= 1e300)) vds_flag(A.err, VDS_ENAN);
+      if (A.imp.st) imp_after_grad(A.imp.st, o[0] / (double)kp.N, o[1], o[2], A.err);
     }
   }
 }
 
 template <int D, int S>
 __global__ void __launch_bounds__(FinCfg<D>::NT) k_dens_finish(PartSrc src, KParams kp, FinArgs A) {
+  FinPtrs P;
+  if (!imp_take(A, false, P)) return;
   using F = FinCfg<D>;
   constexpr int PB = F::PB, SH = D * F::SPL;  // shares of a particle's partial sums
   __shared__ FinShared<D, PB> sh;
@@ -336,11 +428,13 @@ __global__ void __launch_bounds__(FinCfg<D>::NT) k_dens_finish(PartSrc src, KPar
   Sum2 t;
 #pragma unroll
   for (int b = 0; b < SH; ++b) t.add(ps[b][p]);
-  fin_density<D, S, PB, F::NT>(kp, A, base, t.value(), sh);
+  fin_density<D, S, PB, F::NT>(kp, A, P, base, t.value(), sh);
 }
 
 template <int D, int S, int MODE>
 __global__ void __launch_bounds__(FinCfg<D>::NT) k_grad_finish(PartSrc src, KParams kp, FinArgs A) {
+  FinPtrs P;
+  if (!imp_take(A, true, P)) return;
   using F = FinCfg<D>;
   constexpr int PB = F::PB, SPL = F::SPL;
   __shared__ FinShared<D, PB> sh;
@@ -368,7 +462,7 @@ __global__ void __launch_bounds__(FinCfg<D>::NT) k_grad_finish(PartSrc src, KPar
       for (int v = 1; v < SPL; ++v) s[0].add(ps[v][a][p]);
   }
   sum = s[0].value();
-  fin_grad<D, S, MODE, PB, F::NT>(kp, A, base, sum, sh);
+  fin_grad<D, S, MODE, PB, F::NT>(kp, A, P, base, sum, sh);
 }
 
 }  // namespace vds_pair

@@ -70,7 +70,7 @@ struct HasNorm {
 template <int D, int RI, int NT, bool GRAD, int TJK = TJ>
 __global__ void __launch_bounds__(NT)
     k_pair(const float *__restrict__ rec, const float *__restrict__ reci, Sched sc,
-           float2 *__restrict__ part, int *__restrict__ err) {
+           float2 *__restrict__ part, int *__restrict__ err, const ImpState *imp = nullptr) {
   static_assert(TJ % TJK == 0, "j-tiles divide the record padding");
   constexpr int DP = Rec<D>::DP;
   constexpr int ACC = GRAD ? D : 1;
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(NT)
   const int tid = threadIdx.x;
   const long long it0 = (long long)blockIdx.x * sc.items / sc.G;
   const long long it1 = (long long)(blockIdx.x + 1) * sc.items / sc.G;
-  if (it0 >= it1) return;  // uniform over the CTA
+  if (it0 >= it1 || (imp && !imp_due(imp, GRAD))) return;  // uniform over the CTA
 
   if (tid == 0) {
 #pragma unroll
@@ -326,22 +326,79 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) *ticket = 0u;
 }
 
+// Record of y (scaled by c, w = 0, the norm where there is room), or of a
+// padding row.
 template <int D>
-__global__ void k_flow(KParams kp, const float *__restrict__ q, float *__restrict__ qs) {
+__device__ __forceinline__ void put_record(float *rec, int i, float c, const float (&y)[D], bool pad) {
+  constexpr int DP = Rec<D>::DP;
+  float o[DP];
+#pragma unroll
+  for (int d = 0; d < DP; ++d) o[d] = 0.f;
+#pragma unroll
+  for (int d = 0; d < D; ++d) o[d] = pad ? VDS_PAD_COORD : c * y[d];
+  float4 *dst = reinterpret_cast<float4 *>(rec + (size_t)i * DP);
+#pragma unroll
+  for (int v = 0; v < DP / 4; ++v) dst[v] = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
+}
+
+// Start of an implicit step: q* = q + dt kappa q, and the first trial y = q* +
+// d with the previous step's correction d (none in a call's first step).
+template <int D>
+__global__ void k_imp_begin(KParams kp, ImpArgs imp, int Npad, const float *__restrict__ q, float *__restrict__ qs,
+                            float *__restrict__ rec) {
+  const ImpState *s = imp.st;
+  if (s->phase != IMP_READY || s->step >= s->nsteps) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= Npad) return;
+  const bool on = i < kp.N;
+  const float *dcur = s->cur ? imp.d[1] : imp.d[0];
+  float *doth = s->cur ? imp.d[0] : imp.d[1];
+  const bool cold = s->step == 0;
+  float y[D];
+  if (on) {
+#pragma unroll
+    for (int a = 0; a < D; ++a) y[a] = q[(size_t)i * D + a];
+    float f[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const int k = a / kp.s, al = a - k * kp.s;
+      double v = 0.0;
+#pragma unroll
+      for (int b = 0; b < D; ++b)
+        if (b / kp.s == k) v += kp.kappa[al * kp.s + (b - k * kp.s)] * (double)y[b];
+      f[a] = (float)((double)y[a] + kp.dt * v);
+    }
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const float d = cold ? 0.f : dcur[(size_t)i * D + a];
+      qs[(size_t)i * D + a] = f[a];
+      doth[(size_t)i * D + a] = d;
+      y[a] = f[a] + d;
+    }
+  }
+  put_record<D>(rec, i, kp.c, y, !on);
+}
+
+// The next trial point: d[cur] - alpha dir (zero where the step starts cold).
+template <int D>
+__global__ void k_imp_trial(KParams kp, ImpArgs imp, const float *__restrict__ qs, const float *__restrict__ dir,
+                            float *__restrict__ rec) {
+  const ImpState *s = imp.st;
+  if (s->phase != IMP_TRIAL) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= kp.N) return;
+  const float *dcur = s->cur ? imp.d[1] : imp.d[0];
+  float *doth = s->cur ? imp.d[0] : imp.d[1];
+  const float al = (float)s->alpha;
+  const bool zero = s->start != 0;
   float y[D];
 #pragma unroll
-  for (int a = 0; a < D; ++a) y[a] = q[(size_t)i * D + a];
-#pragma unroll
   for (int a = 0; a < D; ++a) {
-    const int k = a / kp.s, al = a - k * kp.s;
-    double v = 0.0;
-#pragma unroll
-    for (int b = 0; b < D; ++b)
-      if (b / kp.s == k) v += kp.kappa[al * kp.s + (b - k * kp.s)] * (double)y[b];
-    qs[(size_t)i * D + a] = (float)((double)y[a] + kp.dt * v);
+    const float d = zero ? 0.f : dcur[(size_t)i * D + a] - al * dir[(size_t)i * D + a];
+    doth[(size_t)i * D + a] = d;
+    y[a] = qs[(size_t)i * D + a] + d;
   }
+  put_record<D>(rec, i, kp.c, y, false);
 }
 
 // ------------------------------------------------------------ host plumbing
@@ -360,7 +417,7 @@ inline int sched_maxseg(const Sched &sc) {
 // i points: the Ni records at reci (the particles themselves unless a query
 // pass); j points: the N particle records in c->rec.
 template <int D, int RI, int NT, bool GRAD, int TJK = TJ>
-int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
+int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci, const ImpState *imp) {
   constexpr int DP = Rec<D>::DP;
   constexpr int ACC = GRAD ? D : 1;
   constexpr int TI = NT * RI;
@@ -390,7 +447,7 @@ int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
   const int pk = GRAD ? PK_GRADIENT : PK_DENSITY;
   VDS_TRY(vds_time_begin(c, pk));
   k_pair<D, RI, NT, GRAD, TJK><<<sc.G, NT, smem, c->stream>>>((const float *)c->rec.ptr, reci, sc,
-                                                                     (float2 *)c->part.ptr, c->err);
+                                                                     (float2 *)c->part.ptr, c->err, imp);
   VDS_CUDA_TRY(cudaGetLastError());
   VDS_TRY(vds_time_end(c, pk));
   ++c->launches;
@@ -416,13 +473,13 @@ int prep_impl(vds_ctx *c, const KParams &kp, const float *base, const float *del
 // not a large fraction of the pass (N = 10000 at D = 9: 200 and 360 items
 // per pass at 256 records).
 template <int D, bool GRAD>
-int launch_pass(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci) {
+int launch_pass(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci, const ImpState *imp = nullptr) {
   constexpr int RI = GRAD ? PairCfg<D>::RI_GRAD : PairCfg<D>::RI_DENS;
   constexpr int NT = GRAD ? PairCfg<D>::NT_GRAD : PairCfg<D>::NT_DENS;
   const long long items = (long long)((Ni + NT * RI - 1) / (NT * RI)) * ((N + TJ - 1) / TJ);
-  if (2 * items < c->num_sms) return launch_pair<D, RI_SMALL, NT_SMALL, GRAD, TJ_SMALL>(c, N, sc, Ni, reci);
-  if (items < 8LL * c->num_sms) return launch_pair<D, RI, NT, GRAD, TJ_SMALL>(c, N, sc, Ni, reci);
-  return launch_pair<D, RI, NT, GRAD>(c, N, sc, Ni, reci);
+  if (2 * items < c->num_sms) return launch_pair<D, RI_SMALL, NT_SMALL, GRAD, TJ_SMALL>(c, N, sc, Ni, reci, imp);
+  if (items < 8LL * c->num_sms) return launch_pair<D, RI, NT, GRAD, TJ_SMALL>(c, N, sc, Ni, reci, imp);
+  return launch_pair<D, RI, NT, GRAD>(c, N, sc, Ni, reci, imp);
 }
 
 // Shapes of the symmetric passes, from sweeps of particles per lane (RI),
@@ -458,7 +515,7 @@ constexpr int SYM_CHUNK_N = 32768;
 // The symmetric pass over the N records at c->rec; done = false (and nothing
 // launched) where its workspace is over the limit or cannot be had.
 template <int D, bool GRAD, int NT, int TJS>
-int launch_sym(vds_ctx *c, int N, Sched &sc, bool &done) {
+int launch_sym(vds_ctx *c, int N, Sched &sc, const ImpState *imp, bool &done) {
   using C = SymCfg<D, GRAD>;
   constexpr int RI = C::RI, TI = NT * RI, ACC = GRAD ? D : 1, MINB = C::MINB128 * 128 / NT;
   constexpr size_t smem = SymSmem<D, RI, NT, GRAD, TJS>::BYTES;
@@ -504,7 +561,7 @@ int launch_sym(vds_ctx *c, int N, Sched &sc, bool &done) {
   const int pk = GRAD ? PK_GRADIENT : PK_DENSITY;
   VDS_TRY(vds_time_begin(c, pk));
   kern<<<sc.G, NT, smem, c->stream>>>((const float *)c->rec.ptr, sc, N, (float2 *)c->part.ptr,
-                                      (float2 *)c->partj.ptr);
+                                      (float2 *)c->partj.ptr, imp);
   VDS_CUDA_TRY(cudaGetLastError());
   VDS_TRY(vds_time_end(c, pk));
   ++c->launches;
@@ -514,16 +571,16 @@ int launch_sym(vds_ctx *c, int N, Sched &sc, bool &done) {
 
 // The pass of the N particles at c->rec against themselves.
 template <int D, bool GRAD>
-int launch_self(vds_ctx *c, int N, PartSrc &src) {
+int launch_self(vds_ctx *c, int N, PartSrc &src, const ImpState *imp) {
   bool done = false;
   if constexpr (GRAD) {
-    if (N >= SYM_LARGE_N) VDS_TRY((launch_sym<D, true, SymCfg<D, true>::NT_LARGE, 32>(c, N, src.sc, done)));
-    else VDS_TRY((launch_sym<D, true, 128, 32>(c, N, src.sc, done)));
+    if (N >= SYM_LARGE_N) VDS_TRY((launch_sym<D, true, SymCfg<D, true>::NT_LARGE, 32>(c, N, src.sc, imp, done)));
+    else VDS_TRY((launch_sym<D, true, 128, 32>(c, N, src.sc, imp, done)));
   } else {
-    if (N >= SYM_CHUNK_N) VDS_TRY((launch_sym<D, false, 128, 64>(c, N, src.sc, done)));
-    else VDS_TRY((launch_sym<D, false, 128, 32>(c, N, src.sc, done)));
+    if (N >= SYM_CHUNK_N) VDS_TRY((launch_sym<D, false, 128, 64>(c, N, src.sc, imp, done)));
+    else VDS_TRY((launch_sym<D, false, 128, 32>(c, N, src.sc, imp, done)));
   }
-  if (!done) VDS_TRY((launch_pass<D, GRAD>(c, N, src.sc, N, (const float *)c->rec.ptr)));
+  if (!done) VDS_TRY((launch_pass<D, GRAD>(c, N, src.sc, N, (const float *)c->rec.ptr, imp)));
   src.i = (const float2 *)c->part.ptr;
   src.j = (const float2 *)c->partj.ptr;
   return VDS_OK;
@@ -597,12 +654,12 @@ int launch_small(vds_ctx *c, const KParams &kp, const FinArgs &A) {
 
 template <int D>
 int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,
-                 const float *ybase, const float *ydelta, const float *qa, const float *qb) {
+                 const float *ybase, const float *ydelta, const float *qa, const float *qb, const ImpArgs *imp) {
   FinArgs A{(float *)c->rec.ptr, rho_out, ybase, ydelta, qa, qb, nullptr, want_energy ? 1 : 0,
-            nullptr, c->ticket + TK_DENS, c->scal, c->err};
+            nullptr, c->ticket + TK_DENS, c->scal, c->err, imp ? *imp : ImpArgs{}};
   if (kp.N < sym_min_n<D>()) return launch_small<D, SM_DENS>(c, kp, A);
   PartSrc src;
-  VDS_TRY((launch_self<D, false>(c, kp.N, src)));
+  VDS_TRY((launch_self<D, false>(c, kp.N, src, A.imp.st)));
   VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
   A.red = (double *)c->red.ptr;
   VDS_TRY((launch_dens_finish<D>(c->stream, src, kp, A)));
@@ -612,8 +669,9 @@ int density_impl(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy
 
 template <int D>
 int grad_impl(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,
-              const float *ydelta, const float *qa, const float *qb, float *q_io) {
-  FinArgs A{(float *)c->rec.ptr, out, ybase, ydelta, qa, qb, q_io, 0, nullptr, c->ticket + TK_GRAD, c->scal, c->err};
+              const float *ydelta, const float *qa, const float *qb, float *q_io, const ImpArgs *imp) {
+  FinArgs A{(float *)c->rec.ptr, out, ybase, ydelta, qa, qb, q_io, 0, nullptr, c->ticket + TK_GRAD, c->scal, c->err,
+            imp ? *imp : ImpArgs{}};
   if (kp.N < sym_min_n<D>()) {
     if (mode == GM_OUT) return launch_small<D, GM_OUT>(c, kp, A);
     if (mode == GM_VEL) return launch_small<D, GM_VEL>(c, kp, A);
@@ -629,7 +687,7 @@ int grad_impl(vds_ctx *c, const KParams &kp, int mode, float *out, const float *
     return VDS_OK;
   }
   PartSrc src;
-  VDS_TRY((launch_self<D, true>(c, kp.N, src)));
+  VDS_TRY((launch_self<D, true>(c, kp.N, src, A.imp.st)));
   VDS_TRY(vds_ensure(c, c->red, fin_red_bytes<D>(kp.N)));
   A.red = (double *)c->red.ptr;
   if (mode == GM_OUT) VDS_TRY((launch_grad_finish<D, GM_OUT>(c->stream, src, kp, A)));
@@ -765,7 +823,7 @@ int rows_grad_impl(vds_ctx *c, const KParams &kp, const float *q, const float *r
   KParams kl = kp;
   kl.N = nrows;
   const FinArgs A{(float *)c->recq.ptr, mode == 0 ? out : nullptr, q + (size_t)row0 * D, nullptr, nullptr, nullptr,
-                  mode == 0 ? nullptr : out, 0, nullptr, nullptr, c->scal, c->err};
+                  mode == 0 ? nullptr : out, 0, nullptr, nullptr, c->scal, c->err, ImpArgs{}};
   if (mode == 0) VDS_TRY((launch_grad_finish<D, GM_OUT>(c->stream, src, kl, A)));
   else VDS_TRY((launch_grad_finish<D, GM_EXPLICIT>(c->stream, src, kl, A)));
   ++c->launches;
@@ -792,8 +850,18 @@ int stress_impl(vds_ctx *c, const KParams &kp, const float *q, double *tau, doub
 }
 
 template <int D>
-int flow_impl(vds_ctx *c, const KParams &kp, const float *q, float *qs) {
-  k_flow<D><<<(kp.N + 255) / 256, 256, 0, c->stream>>>(kp, q, qs);
+int imp_begin_impl(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *q, float *qs) {
+  const int Npad = (kp.N + TJ - 1) / TJ * TJ;
+  VDS_TRY(vds_ensure(c, c->rec, (size_t)Npad * Rec<D>::DP * sizeof(float)));
+  k_imp_begin<D><<<(Npad + 127) / 128, 128, 0, c->stream>>>(kp, imp, Npad, q, qs, (float *)c->rec.ptr);
+  VDS_CUDA_TRY(cudaGetLastError());
+  ++c->launches;
+  return VDS_OK;
+}
+
+template <int D>
+int imp_trial_impl(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs, const float *dir) {
+  k_imp_trial<D><<<(kp.N + 127) / 128, 128, 0, c->stream>>>(kp, imp, qs, dir, (float *)c->rec.ptr);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   return VDS_OK;
@@ -810,18 +878,23 @@ int flow_impl(vds_ctx *c, const KParams &kp, const float *q, float *qs) {
   }                                                                                           \
   int vds_density_##DD(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,       \
                        const float *ybase, const float *ydelta, const float *qa,              \
-                       const float *qb) {                                                     \
-    return vds_pair::density_impl<DD>(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb);    \
+                       const float *qb, const ImpArgs *imp) {                                 \
+    return vds_pair::density_impl<DD>(c, kp, rho_out, want_energy, ybase, ydelta, qa, qb, imp); \
   }                                                                                           \
   int vds_grad_##DD(vds_ctx *c, const KParams &kp, int mode, float *out, const float *ybase,  \
-                    const float *ydelta, const float *qa, const float *qb, float *q_io) {     \
-    return vds_pair::grad_impl<DD>(c, kp, mode, out, ybase, ydelta, qa, qb, q_io);            \
+                    const float *ydelta, const float *qa, const float *qb, float *q_io,       \
+                    const ImpArgs *imp) {                                                     \
+    return vds_pair::grad_impl<DD>(c, kp, mode, out, ybase, ydelta, qa, qb, q_io, imp);       \
   }                                                                                           \
   int vds_stress_##DD(vds_ctx *c, const KParams &kp, const float *q, double *tau, double *qq) { \
     return vds_pair::stress_impl<DD>(c, kp, q, tau, qq);                                      \
   }                                                                                           \
-  int vds_flow_##DD(vds_ctx *c, const KParams &kp, const float *q, float *qs) {               \
-    return vds_pair::flow_impl<DD>(c, kp, q, qs);                                             \
+  int vds_impbegin_##DD(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *q, float *qs) { \
+    return vds_pair::imp_begin_impl<DD>(c, kp, imp, q, qs);                                   \
+  }                                                                                           \
+  int vds_imptrial_##DD(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const float *qs,    \
+                        const float *dir) {                                                   \
+    return vds_pair::imp_trial_impl<DD>(c, kp, imp, qs, dir);                                 \
   }                                                                                           \
   int vds_query_##DD(vds_ctx *c, const KParams &kp, const float *q, const float *y, int M,     \
                      float *f) {                                                              \

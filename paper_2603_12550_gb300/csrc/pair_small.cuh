@@ -30,6 +30,8 @@ __global__ void __launch_bounds__(NT) k_small(const float *rec, KParams kp, FinA
   __shared__ float red[W][ACC][PB];
   const int tid = threadIdx.x, w = tid >> 5, li = tid & 7, lj = (tid >> 3) & 3;
   const int base = blockIdx.x * PB, N = kp.N;
+  FinPtrs P;
+  if (!imp_take(A, GRAD, P)) return;
   float xi[RI][D], wi[RI], acc[RI][ACC];
 #pragma unroll
   for (int k = 0; k < RI; ++k) {
@@ -87,8 +89,8 @@ __global__ void __launch_bounds__(NT) k_small(const float *rec, KParams kp, FinA
   if (a < D)
 #pragma unroll
     for (int x = 0; x < W; ++x) s.add(make_float2(red[x][GRAD ? a : 0][p], 0.f));
-  if constexpr (GRAD) fin_grad<D, S, MODE, PB, NT>(kp, A, base, s.value(), sh);
-  else fin_density<D, S, PB, NT>(kp, A, base, s.value(), sh);
+  if constexpr (GRAD) fin_grad<D, S, MODE, PB, NT>(kp, A, P, base, s.value(), sh);
+  else fin_density<D, S, PB, NT>(kp, A, P, base, s.value(), sh);
 }
 
 }  // namespace vds_pair

@@ -81,7 +81,8 @@ struct SymSmem {
 
 template <int D, int RI, int NT, int MINB, bool GRAD, int TJS>
 __global__ void __launch_bounds__(NT, MINB)
-    k_sym(const float *__restrict__ rec, Sched sc, int N, float2 *__restrict__ part, float2 *__restrict__ partj) {
+    k_sym(const float *__restrict__ rec, Sched sc, int N, float2 *__restrict__ part, float2 *__restrict__ partj,
+          const ImpState *imp) {
   using L = SymSmem<D, RI, NT, GRAD, TJS>;
   constexpr int DP = Rec<D>::DP, VG = DP / 4, V = L::V, ACC = L::ACC, W = NT / 32, TI = NT * RI;
   constexpr int CPT = TI / TJS;
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(NT, MINB)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long it0 = (long long)blockIdx.x * sc.items / sc.G;
   const long long it1 = (long long)(blockIdx.x + 1) * sc.items / sc.G;
-  if (it0 >= it1) return;  // uniform over the CTA
+  if (it0 >= it1 || (imp && !imp_due(imp, GRAD))) return;  // uniform over the CTA
 
   // i-tile and chunk of the first item
   int t = 0;

@@ -209,7 +209,7 @@ void vds_destroy(vds_ctx *c) {
   DeviceGuard g(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
-  DevBuf *bufs[] = {&c->rec, &c->rec2, &c->recq, &c->part, &c->partj, &c->red, &c->vecs, &c->gbuf, &c->ubuf, &c->dtbuf};
+  DevBuf *bufs[] = {&c->rec, &c->rec2, &c->recq, &c->part, &c->partj, &c->red, &c->vecs, &c->imp, &c->gbuf, &c->ubuf, &c->dtbuf};
   for (DevBuf *b : bufs)
     if (b->ptr) cudaFree(b->ptr);
   if (c->err) cudaFree(c->err);
@@ -393,78 +393,61 @@ static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
   return st != VDS_OK ? st : sst;
 }
 
-// Implicit Euler step as the minimiser of J (see vds.h).  y = q* + d is
-// carried through d = y - q*, which keeps the dissipation term of J accurate
-// in FP32.
+// Implicit Euler steps as minimisers of J (see vds.h).  y = q* + d is carried
+// through d = y - q*, which keeps the dissipation term of J accurate in FP32.
+// Each step starts from y = q* + (the previous step's solution - its q*): the
+// correction varies slowly between steps, so the minimiser usually needs one
+// gradient evaluation fewer; from q* itself in the first step of a call or
+// when that start leaves the FENE domain.
+//
+// The minimiser runs on the device (ImpState, set by the passes' epilogues),
+// so that no evaluation waits for the host: read back after each of about
+// seven evaluations, the 2D dumbbell at N = 512 took 300-400 us a step, two
+// thirds of it host round trips.  The host enqueues rounds of (trial point,
+// density, gradient) without looking; those that are not due return at once
+// (about 2 us).  Most steps need two gradients: two rounds per step are
+// enqueued, a step that needs more goes on in the rounds meant for the next,
+// and what is missing at the end is enqueued then.
 static int step_implicit(vds_ctx *c, float *q, const KParams &kp, const vds_params *p, int nsteps,
                          int *iters_out) {
   const size_t nd = (size_t)kp.N * kp.D;
   VDS_TRY(vds_ensure(c, c->vecs, 4 * nd * sizeof(float)));
-  float *qs = vec(c, 0, nd), *d0 = vec(c, 1, nd), *d1 = vec(c, 2, nd), *dir = vec(c, 3, nd);
-  for (int n = 0; n < nsteps; ++n) {
-    VDS_TRY(pass_flow(c, kp, q, qs));
-    // start from y = q* + (the previous step's solution - its q*): the
-    // correction varies slowly between steps, so the minimiser usually needs
-    // one gradient evaluation fewer; q* itself for the first step of a call or
-    // when that start leaves the FENE domain
-    double J = 0.0;
-    bool warm = n > 0;
-    for (;;) {
-      if (!warm) VDS_CUDA_TRY(cudaMemsetAsync(d0, 0, nd * sizeof(float), c->stream));
-      VDS_TRY(pass_prep(c, kp, qs, d0, nullptr, 0.f, nullptr));
-      VDS_TRY(pass_density(c, kp, nullptr, true, qs, d0, d0, nullptr));
-      const int st = read_scalars(c);
-      if (st == VDS_EDOMAIN && warm) {
-        warm = false;
-        continue;
-      }
-      VDS_TRY(st);
-      J = c->h_scal[SC_E];
-      break;
+  float *qs = vec(c, 0, nd), *dir = vec(c, 3, nd);
+  VDS_TRY(vds_ensure(c, c->imp, sizeof(ImpState) + (size_t)nsteps * sizeof(int)));
+  ImpState s = {};
+  s.J = INFINITY;
+  s.tol = p->tol;
+  s.jfloor = p->jfloor;
+  s.max_iter = p->max_iter;
+  s.nsteps = nsteps;
+  ImpArgs imp;
+  imp.st = (ImpState *)c->imp.ptr;
+  imp.d[0] = vec(c, 1, nd);
+  imp.d[1] = vec(c, 2, nd);
+  int *iters = (int *)(imp.st + 1);
+  VDS_CUDA_TRY(cudaMemcpyAsync(imp.st, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
+  auto one_step = [&](int rounds) -> int {
+    VDS_TRY(imp_begin(c, kp, imp, q, qs));
+    for (int r = 0; r < rounds; ++r) {
+      if (r) VDS_TRY(imp_trial(c, kp, imp, qs, dir));
+      VDS_TRY(pass_density(c, kp, nullptr, true, qs, nullptr, nullptr, nullptr, &imp));
+      VDS_TRY(pass_grad(c, kp, GM_IMPLICIT_DIR, dir, qs, nullptr, nullptr, nullptr, nullptr, &imp));
     }
-    int it = 0;
-    bool converged = false;
-    while (it < p->max_iter) {
-      ++it;
-      VDS_TRY(pass_grad(c, kp, GM_IMPLICIT_DIR, dir, qs, d0, nullptr, nullptr, nullptr));
-      VDS_TRY(read_scalars(c));
-      const double dec = c->h_scal[SC_DEC], dmax = c->h_scal[SC_DMAX], ymax = c->h_scal[SC_YMAX];
-      if (dmax <= p->tol * (1.0 + ymax)) {
-        VDS_TRY(pass_prep(c, kp, qs, d0, dir, 1.f, d1));
-        float *t = d0;
-        d0 = d1;
-        d1 = t;
-        converged = true;
-        break;
-      }
-      double alpha = 1.0, Jn = 0.0;
-      bool acc = false;
-      for (int ls = 0; ls <= 30; ++ls) {
-        VDS_TRY(pass_prep(c, kp, qs, d0, dir, (float)alpha, d1));
-        VDS_TRY(pass_density(c, kp, nullptr, true, qs, d1, d1, nullptr));
-        const int st = read_scalars(c);
-        if (st != VDS_OK && st != VDS_EDOMAIN) return st;
-        Jn = c->h_scal[SC_E];
-        if (st == VDS_OK && Jn <= J - 1e-4 * alpha * dec + p->jfloor * (1.0 + fabs(J))) {
-          acc = true;
-          break;
-        }
-        alpha *= 0.5;
-      }
-      if (!acc) return VDS_ENOCONV;
-      float *t = d0;
-      d0 = d1;
-      d1 = t;
-      J = Jn;
-    }
-    if (iters_out) iters_out[n] = it;
-    VDS_TRY(pass_axpy(c, (int)nd, qs, d0, q));
-    if (!converged) {
-      VDS_TRY(vds_sync_status(c));
-      return VDS_ENOCONV;
+    VDS_TRY(imp_trial(c, kp, imp, qs, dir));  // for a step that goes on
+    return imp_end(c, kp, imp, qs, dir, q, iters);
+  };
+  for (bool first = true;; first = false) {
+    // at most this many steps ahead of the host
+    const int ahead = nsteps - s.step < 64 ? nsteps - s.step : 64;
+    for (int k = 0; k < ahead; ++k) VDS_TRY(one_step(kp.N > 16384 ? 2 : first && k > 0 ? 3 : 4));
+    VDS_CUDA_TRY(cudaMemcpyAsync(&s, imp.st, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
+    const int st = vds_sync_status(c);
+    if (st != VDS_OK || s.phase == IMP_STOP || s.step >= nsteps) {
+      if (iters_out && s.step > 0)
+        VDS_CUDA_TRY(cudaMemcpy(iters_out, iters, (size_t)s.step * sizeof(int), cudaMemcpyDeviceToHost));
+      return st != VDS_OK ? st : s.status;
     }
   }
-  return vds_sync_status(c);
 }
 
 int vds_step(vds_ctx *c, float *q, int N, int D, const vds_params *p, int nsteps, int *iters_out) {

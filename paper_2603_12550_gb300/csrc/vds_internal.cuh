@@ -217,6 +217,7 @@ struct vds_ctx {
   DevBuf partj;    // j-side partial sums of the symmetric passes (FP64)
   DevBuf red;      // block partials of reductions (FP64)
   DevBuf vecs;     // minimiser vectors / scratch (FP32)
+  DevBuf imp;      // minimiser state and iteration counts
   DevBuf gbuf;     // Gram / projection partials (FP64)
   DevBuf ubuf;     // reduced-order scratch (refresh outputs, reduced state)
   DevBuf dtbuf;    // tensor-core density: operand images and split partials
