@@ -11,12 +11,15 @@
  * velocity gradient kappa_e; the other parameters (springs, kBT, zeta, dt,
  * scheme, tolerances) are shared.  Same status codes as vds.h.
  *
- * Work distribution: one persistent kernel per pair pass pops work items
+ * Work distribution: a persistent kernel per pair pass pops work items
  * (e, i-tile) from a queue in longest-processing-time order -- cost N_e
  * descending, then e ascending, then tile ascending -- with an atomic
  * counter; an item covers all j of its ensemble, so every particle's sums are
  * formed by one CTA in a fixed order and the results do not depend on the
- * schedule.
+ * schedule.  Ensembles of 2048 particles and more are taken over unordered
+ * pairs instead, in units of their own (an i-tile against up to 1024 later
+ * particles) whose sums have their own places and are added in a fixed order;
+ * the queue lists every ensemble's items all the same.
  */
 #ifndef VDS_BATCH_H
 #define VDS_BATCH_H
@@ -91,7 +94,8 @@ VDS_API int vds_convect(vds_ctx *ctx, const float *q_in, float *q_out, int nx, i
  * per CTA with 2 << (k & 1) particles per thread, so a work item's i-tile is
  * 256, 512, 512 or 1024 particles.  The j-tiles and the order of every sum
  * are the same in all of them, so results are bit-identical across configs;
- * only the queue (its items follow the tile) and the speed change.  A batch
+ * only the queue (its items follow the tile) and the speed change.  Ensembles
+ * over unordered pairs have one shape and do not depend on the config.  A batch
  * starts in config 1 for D <= 6 and config 0 otherwise.
  *
  * vds_batch_autotune times one density and one gradient pass of every

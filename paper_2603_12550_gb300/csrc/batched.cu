@@ -1,12 +1,16 @@
 // batched.cu -- many independent VDS ensembles of uneven size advanced
 // together (include/vds_batch.h).
 //
-// One persistent pair kernel per pass: each CTA pops (ensemble, i-tile) work
-// items, in longest-processing-time order, from an atomic counter and streams
-// all j-tiles of that ensemble through a shared-memory ring filled by TMA bulk
-// copies.  An item covers the whole j range, so every particle's sums are
-// formed by one CTA in a fixed order (plain FP32 inside a j-tile, Kahan across
-// tiles): results are independent of which CTA took which item.
+// Persistent pair kernels per pass.  Ensembles of BSYM_MIN_N particles and more
+// go over unordered pairs (k_bsym): units of one i-tile against up to BSYM_RUN
+// j-chunks, in longest-processing-time order from an atomic counter, each
+// leaving its sums in its own place; k_bgather adds a particle's in a fixed
+// order.  The units of an ensemble depend on its size alone.  Smaller ones go
+// over ordered pairs (k_bpair): (ensemble, i-tile) items of the chosen shape
+// that stream all j-tiles of the ensemble through a shared-memory ring filled
+// by TMA bulk copies, every particle's sums formed by one CTA (plain FP32 inside
+// a j-tile, Kahan across tiles).  Either way results are independent of which
+// CTA took what.
 //
 // Implicit steps run every ensemble's minimiser (the single-ensemble
 // algorithm of vds_step, scheme 1) in lockstep rounds.  Per-ensemble state
@@ -24,7 +28,7 @@
 #include <vector>
 
 #include "../../include/vds_batch.h"
-#include "vds_internal.cuh"
+#include "pair_impl.cuh"
 
 namespace {
 
@@ -211,6 +215,132 @@ __global__ void __launch_bounds__(NT)
     }
     gtile += (Ne + BTJ - 1) / BTJ;
   }
+}
+
+// ------------------------------------------- unordered pairs, large ensembles
+
+// Ensembles from this size on (two i-tiles or more of every D): N = 2048 in two
+// tiles of 1024 is three tile pairs' work where the ordered form has four.
+constexpr int BSYM_MIN_N = 2048;
+constexpr int BSYM_TJS = 32, BSYM_NT = 128;
+constexpr int BSYM_RUN = 32;                           // j-chunks per unit
+constexpr long long BSYM_MAX_FLOAT2 = (long long)1 << 29;  // workspace: 4 GiB
+
+template <int D>
+struct BSymCfg {
+  static constexpr int RI = vds_pair::SymCfg<D, true>::RI, MINB = vds_pair::SymCfg<D, true>::MINB128;
+  static constexpr int TI = BSYM_NT * RI, CPT = TI / BSYM_TJS;
+  static constexpr size_t SMEM = vds_pair::SymSmem<D, RI, BSYM_NT, true, BSYM_TJS>::BYTES;
+};
+
+struct BUnit {
+  int e, t, ca, cb;
+  int run;  // its place among the i sums
+  int pad;
+};
+// Per ensemble: first entry of its i-tiles in the table of runs, first element
+// of its j sums (in columns, times D), j-chunks; tiles < 0: not taken here.
+struct BEns {
+  int tile0, ntile, nchunk, pad;
+  long long jcol;
+};
+
+__host__ __device__ __forceinline__ Sched bsym_sched(int nchunk, int cpt, int TI) {
+  Sched sc = {};
+  sc.nchunk = nchunk;
+  sc.cpt = cpt;
+  sc.TI = TI;
+  return sc;
+}
+
+// mode as k_bpair.
+template <int D>
+__global__ void __launch_bounds__(BSYM_NT, BSymCfg<D>::MINB)
+    k_bsym(const float *__restrict__ rec, const long long *__restrict__ off, const int *__restrict__ sizes,
+           const BUnit *__restrict__ units, int nunits, const BEns *__restrict__ ens, unsigned *counter, int mode,
+           const BState *__restrict__ st, float2 *__restrict__ ipart, float2 *__restrict__ jpart) {
+  using C = BSymCfg<D>;
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  __shared__ int s_unit;
+  for (;;) {
+    if (threadIdx.x == 0) s_unit = (int)atomicAdd(counter, 1u);
+    __syncthreads();
+    const int u = s_unit;
+    __syncthreads();
+    if (u >= nunits) return;
+    const BUnit w = units[u];
+    bool grad = mode == 1;
+    if (mode == 2) {
+      const int ph = st[w.e].phase;
+      if (ph != ST_TRIAL && ph != ST_GRAD) continue;
+      grad = ph == ST_GRAD;
+    }
+    const float *r = rec + (size_t)off[w.e] * Rec<D>::DP;
+    const BEns E = ens[w.e];
+    const Sched sc = bsym_sched(E.nchunk, C::CPT, C::TI);
+    float2 *ip = ipart + (size_t)w.run * D * C::TI;
+    float2 *jp = jpart + (size_t)E.jcol * D;
+    const size_t jr = (size_t)sched_jrow(w.t, sc);
+    const long long ncol = sched_jcols(w.t, sc);
+    if (grad)
+      vds_pair::sym_run<D, C::RI, BSYM_NT, true, BSYM_TJS>(r, sizes[w.e], w.t, w.ca, w.cb, sm_raw, ip, jp + jr * D,
+                                                           ncol);
+    else
+      vds_pair::sym_run<D, C::RI, BSYM_NT, false, BSYM_TJS>(r, sizes[w.e], w.t, w.ca, w.cb, sm_raw, ip, jp + jr, ncol);
+    __syncthreads();
+  }
+}
+
+// acc[i][a] (acc[i][0] for a density) of 32 particles per CTA, from the units'
+// sums: the i side's runs of the particle's tile, then the rows that earlier
+// tiles left, in order.  blocks[b]: ensemble and first particle.
+template <int D>
+__global__ void __launch_bounds__(32 * D)
+    k_bgather(const int2 *__restrict__ blocks, const long long *__restrict__ off, const int *__restrict__ sizes,
+              const BEns *__restrict__ ens, const int *__restrict__ runs, int mode, const BState *__restrict__ st,
+              const float2 *__restrict__ ipart, const float2 *__restrict__ jpart, double *__restrict__ acc) {
+  using C = BSymCfg<D>;
+  __shared__ float2 ps[D][32];
+  const int2 w = blocks[blockIdx.x];
+  bool grad = mode == 1;
+  if (mode == 2) {
+    const int ph = st[w.x].phase;
+    if (ph != ST_TRIAL && ph != ST_GRAD) return;
+    grad = ph == ST_GRAD;
+  }
+  const int p = threadIdx.x & 31, a = threadIdx.x >> 5, i = w.y + p;
+  const BEns E = ens[w.x];
+  const Sched sc = bsym_sched(E.nchunk, C::CPT, C::TI);
+  const bool on = i < sizes[w.x];
+  const int t = i / C::TI, il = i - t * C::TI;
+  const int r0 = on ? runs[E.tile0 + t] : 0, nr = on ? runs[E.tile0 + t + 1] - r0 : 0, n = on ? nr + t : 0;
+  const float2 *jp = jpart + (size_t)E.jcol * D;
+  auto get = [&](int x, int aa, int accs) {
+    if (x < nr) return ipart[(size_t)(r0 + x) * D * C::TI + (size_t)aa * C::TI + il];
+    const int r = x - nr;
+    return jp[(size_t)sched_jrow(r, sc) * accs + (size_t)aa * sched_jcols(r, sc) + (i - (r + 1) * C::TI)];
+  };
+  vds_pair::Sum2 s;
+  if (grad) {
+    vds_pair::Sum2 q[4];
+    for (int x = 0; x < n; x += 4)
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        if (x + v < n) q[v].add(get(x + v, a, D));
+    s = q[0];
+#pragma unroll
+    for (int v = 1; v < 4; ++v) s.add(make_float2(q[v].s, q[v].c));
+    if (on) acc[(size_t)(off[w.x] + i) * D + a] = s.value();
+    return;
+  }
+  for (int x = a; x < n; x += D) s.add(get(x, 0, 1));
+  ps[a][p] = make_float2(s.s, s.c);
+  __syncthreads();
+  if (a || !on) return;
+  vds_pair::Sum2 q;
+#pragma unroll
+  for (int b = 0; b < D; ++b) q.add(ps[b][p]);
+  acc[(size_t)(off[w.x] + i) * D] = q.value();
 }
 
 // ------------------------------------------------------ per-particle kernels
@@ -638,6 +768,14 @@ struct vds_batch {
   float *rec = nullptr, *qs = nullptr, *dA = nullptr, *dB = nullptr, *dir = nullptr, *dprev = nullptr;
   double *acc = nullptr, *contrib = nullptr, *eout = nullptr;
   size_t smem = 0;
+  // unordered pairs: units, runs and blocks of the large ensembles, their sums
+  int nord = 0, nunits = 0, nblocks = 0, sym_grid = 0;
+  std::vector<char> sym;  // per ensemble
+  BUnit *d_units = nullptr;
+  BEns *d_bens = nullptr;
+  int *d_runs = nullptr;
+  int2 *d_blocks = nullptr;
+  float2 *ipart = nullptr, *jpart = nullptr;
   cudaGraphExec_t round_exec = nullptr;
   cudaGraph_t round_graph = nullptr;
   cudaStream_t graph_stream = nullptr;  // stream the round graph was captured for
@@ -648,7 +786,8 @@ namespace {
 
 template <int D, int RI, int NT>
 int b_launch_cfg(vds_ctx *c, vds_batch *b, int mode) {
-  k_bpair<D, RI, NT><<<b->grid, NT, b->smem, c->stream>>>(b->rec, b->d_off, b->d_sizes, b->d_queue, b->nitems,
+  if (!b->nord) return VDS_OK;
+  k_bpair<D, RI, NT><<<b->grid, NT, b->smem, c->stream>>>(b->rec, b->d_off, b->d_sizes, b->d_queue, b->nord,
                                                            b->d_counter, mode, b->d_st, b->acc, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
   return VDS_OK;
@@ -656,8 +795,18 @@ int b_launch_cfg(vds_ctx *c, vds_batch *b, int mode) {
 
 template <int D>
 int b_launch_pair(vds_ctx *c, vds_batch *b, int mode) {
-  VDS_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), c->stream));
+  VDS_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(unsigned), c->stream));
   VDS_TRY(vds_time_begin(c, mode == 1 ? PK_GRADIENT : PK_DENSITY));
+  if (b->nunits) {
+    k_bsym<D><<<b->sym_grid, BSYM_NT, BSymCfg<D>::SMEM, c->stream>>>(b->rec, b->d_off, b->d_sizes, b->d_units,
+                                                                     b->nunits, b->d_bens, b->d_counter + 1, mode,
+                                                                     b->d_st, b->ipart, b->jpart);
+    VDS_CUDA_TRY(cudaGetLastError());
+    k_bgather<D><<<b->nblocks, 32 * D, 0, c->stream>>>(b->d_blocks, b->d_off, b->d_sizes, b->d_bens, b->d_runs, mode,
+                                                       b->d_st, b->ipart, b->jpart, b->acc);
+    VDS_CUDA_TRY(cudaGetLastError());
+    c->launches += 2;
+  }
   switch (b->cfg) {
     case 0: VDS_TRY((b_launch_cfg<D, kCfgRI[0], kCfgNT[0]>(c, b, mode))); break;
     case 1: VDS_TRY((b_launch_cfg<D, kCfgRI[1], kCfgNT[1]>(c, b, mode))); break;
@@ -665,7 +814,7 @@ int b_launch_pair(vds_ctx *c, vds_batch *b, int mode) {
     default: VDS_TRY((b_launch_cfg<D, kCfgRI[3], kCfgNT[3]>(c, b, mode))); break;
   }
   VDS_TRY(vds_time_end(c, mode == 1 ? PK_GRADIENT : PK_DENSITY));
-  ++c->launches;
+  if (b->nord) ++c->launches;
   return VDS_OK;
 }
 
@@ -752,7 +901,69 @@ void b_build_queue(vds_batch *b) {
     b->items[2 * k] = its[k].e;
     b->items[2 * k + 1] = its[k].t;
   }
-  if (b->grid > b->nitems) b->grid = b->nitems;
+}
+
+// The units of the ensembles of BSYM_MIN_N particles and more, largest first,
+// and the workspace of their sums; ensembles for which the workspace is over
+// its limit or cannot be had stay with the ordered items.
+template <int D>
+int b_setup_sym(vds_ctx *c, vds_batch *b) {
+  using C = BSymCfg<D>;
+  std::vector<BUnit> units;
+  std::vector<BEns> ens(b->E, BEns{0, -1, 0, 0, 0});
+  std::vector<int> runs;
+  std::vector<int2> blocks;
+  long long jcol = 0;
+  int nrun = 0;
+  b->sym.assign(b->E, 0);
+  for (int e = 0; e < b->E; ++e) {
+    const int N = b->sizes[e];
+    if (N < BSYM_MIN_N) continue;
+    const int nchunk = (N + BSYM_TJS - 1) / BSYM_TJS, ntile = (N + C::TI - 1) / C::TI;
+    const Sched sc = bsym_sched(nchunk, C::CPT, C::TI);
+    long long er = 0;
+    for (int t = 0; t < ntile; ++t) er += (nchunk - t * C::CPT + BSYM_RUN - 1) / BSYM_RUN;
+    const long long ej = sched_jrow(ntile - 1, sc);
+    if ((jcol + ej + (nrun + er) * C::TI) * D > BSYM_MAX_FLOAT2) continue;
+    b->sym[e] = 1;
+    ens[e] = BEns{(int)runs.size(), ntile, nchunk, 0, jcol};
+    for (int t = 0; t < ntile; ++t) {
+      runs.push_back(nrun);
+      for (int ca = t * C::CPT; ca < nchunk; ca += BSYM_RUN)
+        units.push_back(BUnit{e, t, ca, std::min(nchunk, ca + BSYM_RUN), nrun++, 0});
+    }
+    runs.push_back(nrun);
+    jcol += ej;
+    for (int i = 0; i < N; i += 32) blocks.push_back(make_int2(e, i));
+  }
+  if (units.empty()) return VDS_OK;
+  std::stable_sort(units.begin(), units.end(), [](const BUnit &x, const BUnit &y) { return x.cb - x.ca > y.cb - y.ca; });
+  VDS_CUDA_TRY(cudaFuncSetAttribute(k_bsym<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+  int occ = 0;
+  VDS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bsym<D>, BSYM_NT, C::SMEM));
+  const long long grid = (long long)c->num_sms * (occ > 0 ? occ : 1);
+  auto put = [&](void **dst, const void *src, size_t bytes) -> cudaError_t {
+    const cudaError_t e = cudaMalloc(dst, bytes);
+    return e != cudaSuccess || !src ? e : cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
+  };
+  cudaError_t ce = put((void **)&b->d_units, units.data(), units.size() * sizeof(BUnit));
+  if (ce == cudaSuccess) ce = put((void **)&b->d_bens, ens.data(), ens.size() * sizeof(BEns));
+  if (ce == cudaSuccess) ce = put((void **)&b->d_runs, runs.data(), runs.size() * sizeof(int));
+  if (ce == cudaSuccess) ce = put((void **)&b->d_blocks, blocks.data(), blocks.size() * sizeof(int2));
+  if (ce == cudaSuccess) ce = put((void **)&b->ipart, nullptr, (size_t)nrun * C::TI * D * sizeof(float2));
+  if (ce == cudaSuccess) ce = put((void **)&b->jpart, nullptr, ((size_t)jcol * D + 1) * sizeof(float2));
+  if (ce == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    b->sym.assign(b->E, 0);  // all ensembles over ordered pairs
+    if (b->ipart) cudaFree(b->ipart);
+    b->ipart = nullptr;
+    return VDS_OK;
+  }
+  VDS_CUDA_TRY(ce);
+  b->nunits = (int)units.size();
+  b->nblocks = (int)blocks.size();
+  b->sym_grid = (int)(grid < b->nunits ? grid : b->nunits);
+  return VDS_OK;
 }
 
 void b_drop_graph(vds_batch *b) {
@@ -775,8 +986,14 @@ int b_apply_config(vds_ctx *c, vds_batch *b, int cfg) {
   VDS_TRY(st);
   b_build_queue(b);
   if (b->nitems > b->max_items) return VDS_EARG;
-  VDS_CUDA_TRY(cudaMemcpyAsync(b->d_queue, b->items.data(), sizeof(int2) * b->nitems, cudaMemcpyHostToDevice,
-                               c->stream));
+  // what k_bpair takes of the queue: the items of the ensembles over ordered pairs
+  std::vector<int2> ord;
+  for (int k = 0; k < b->nitems; ++k)
+    if (!b->sym[b->items[2 * k]]) ord.push_back(make_int2(b->items[2 * k], b->items[2 * k + 1]));
+  b->nord = (int)ord.size();
+  if (b->grid > b->nord) b->grid = b->nord;
+  if (b->nord)
+    VDS_CUDA_TRY(cudaMemcpyAsync(b->d_queue, ord.data(), sizeof(int2) * b->nord, cudaMemcpyHostToDevice, c->stream));
   VDS_CUDA_TRY(cudaStreamSynchronize(c->stream));
   b_drop_graph(b);
   return VDS_OK;
@@ -851,7 +1068,7 @@ int b_step(vds_ctx *c, vds_batch *b, float *q, int nsteps, int *iters_out, int s
     b->graph_stream = c->stream;
     b->graph_q = q;
   }
-  const int round_launches = 4;
+  const int round_launches = 3 + (b->nunits ? 2 : 0) + (b->nord ? 1 : 0);
   const int max_rounds = 32 * (b->cm.max_iter + 1) + 4;
   std::vector<BState> hs(b->E);
   int status = VDS_OK;
@@ -951,7 +1168,8 @@ void vds_batch_free(vds_batch *b) {
   Dev dg(b->device);
   b_drop_graph(b);
   void *ptrs[] = {b->d_off, b->d_sizes, b->d_ens, b->d_active, b->d_queue, b->d_counter, b->d_ep, b->d_st,
-                  b->rec, b->qs, b->dA, b->dB, b->dir, b->dprev, b->acc, b->contrib, b->eout};
+                  b->rec, b->qs, b->dA, b->dB, b->dir, b->dprev, b->acc, b->contrib, b->eout,
+                  b->d_units, b->d_bens, b->d_runs, b->d_blocks, b->ipart, b->jpart};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (b->h_active) cudaFreeHost(b->h_active);
@@ -1019,7 +1237,7 @@ int vds_batch_create(vds_ctx *c, int E, const int *sizes, int D, const vds_param
   A((void **)&b->d_ens, sizeof(int) * tot);
   A((void **)&b->d_active, sizeof(int));
   A((void **)&b->d_queue, sizeof(int2) * b->max_items);
-  A((void **)&b->d_counter, sizeof(unsigned));
+  A((void **)&b->d_counter, 2 * sizeof(unsigned));
   A((void **)&b->d_ep, sizeof(EParam) * E);
   A((void **)&b->d_st, sizeof(BState) * E);
   A((void **)&b->rec, sizeof(float) * (size_t)tot * Rec<12>::DP);
@@ -1041,7 +1259,10 @@ int vds_batch_create(vds_ctx *c, int E, const int *sizes, int D, const vds_param
     vds_batch_free(b);
     return ce == cudaErrorMemoryAllocation ? VDS_ENOMEM : VDS_ECUDA;
   }
-  const int st = b_apply_config(c, b, default_config(D));
+#define SYM(DD) b_setup_sym<DD>(c, b)
+  int st = [&]() -> int { VDS_BATCH_D(D, SYM) }();
+#undef SYM
+  if (st == VDS_OK) st = b_apply_config(c, b, default_config(D));
   if (st != VDS_OK) {
     vds_batch_free(b);
     return st;

@@ -79,10 +79,16 @@ struct SymSmem {
   static constexpr size_t BYTES = TILE + JS + KAHAN;
 };
 
-template <int D, int RI, int NT, int MINB, bool GRAD, int TJS>
-__global__ void __launch_bounds__(NT, MINB)
-    k_sym(const float *__restrict__ rec, Sched sc, int N, float2 *__restrict__ part, float2 *__restrict__ partj,
-          const ImpState *imp) {
+// The pairs of i-tile t (TI particles) with the chunks [ca, cb), from the
+// tile's own first chunk on, of the N records at rec: the i side's sums into
+// ipart ([component][TI]), the j side's into jrow ([component][ncol], column 0
+// the first record after the tile).  All threads of the CTA; sm_raw holds
+// SymSmem::BYTES.  What it writes depends on nothing but the records, t, ca
+// and cb.
+template <int D, int RI, int NT, bool GRAD, int TJS>
+__device__ __forceinline__ void sym_run(const float *__restrict__ rec, int N, int t, int ca, int cb,
+                                        unsigned char *sm_raw, float2 *__restrict__ ipart, float2 *__restrict__ jrow,
+                                        long long ncol) {
   using L = SymSmem<D, RI, NT, GRAD, TJS>;
   constexpr int DP = Rec<D>::DP, VG = DP / 4, V = L::V, ACC = L::ACC, W = NT / 32, TI = NT * RI;
   constexpr int CPT = TI / TJS;
@@ -91,49 +97,53 @@ __global__ void __launch_bounds__(NT, MINB)
   constexpr int FOLD = (GRAD && NT > 128 ? 128 : 64) / TJS;
   using JS = JSlots<ACC, TJS>;
   static_assert(TI % TJS == 0 && TJS % 32 == 0 && 256 % TJS == 0, "tile shapes");
-  extern __shared__ __align__(128) unsigned char sm_raw[];
   float4 *tile = reinterpret_cast<float4 *>(sm_raw);                   // [2][V][TJS]
   float *js = reinterpret_cast<float *>(sm_raw + L::TILE);             // [2][W][ACC x TJS]
   float *ks = reinterpret_cast<float *>(sm_raw + L::TILE + L::JS);     // [RI x ACC][NT] sums
   float *kc = ks + (size_t)RI * ACC * NT;                              // ... and compensations
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long it0 = (long long)blockIdx.x * sc.items / sc.G;
-  const long long it1 = (long long)(blockIdx.x + 1) * sc.items / sc.G;
-  if (it0 >= it1 || (imp && !imp_due(imp, GRAD))) return;  // uniform over the CTA
-
-  // i-tile and chunk of the first item
-  int t = 0;
-  {
-    int lo = 0, hi = sc.n_itiles;
-    while (hi - lo > 1) {
-      const int m = (lo + hi) >> 1;
-      if (sched_start(m, sc) <= it0) lo = m;
-      else hi = m;
-    }
-    t = lo;
-  }
-  int c = t * CPT + (int)(it0 - sched_start(t, sc));
 
   auto stage = [&](int chunk, int buf) {
     const float4 *src = reinterpret_cast<const float4 *>(rec) + (size_t)chunk * TJS * VG;
     float4 *dst = tile + buf * V * TJS;
+    const int n = N - chunk * TJS;
 #pragma unroll
     for (int x0 = 0; x0 < V * TJS; x0 += NT) {
       const int x = x0 + tid;
       if (V * TJS % NT == 0 || x < V * TJS) {
         const int j = x / V, v = x - j * V;
-        cp_async16(dst + v * TJS + j, src + (size_t)j * VG + v);
+        if (j < n) {
+          cp_async16(dst + v * TJS + j, src + (size_t)j * VG + v);
+        } else {  // past the last particle: no kernel value, no weight
+          float o[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) o[k] = 4 * v + k < D ? VDS_PAD_COORD : 0.f;
+          dst[v * TJS + j] = make_float4(o[0], o[1], o[2], o[3]);
+        }
       }
     }
   };
 
-  stage(c, 0);
+  stage(ca, 0);
 
   float xi[RI][D], wi[RI], acc[RI][ACC];
-  int cur = -1, nf = 0;
+  int nf = 0;
   const int i0 = warp * 32 * RI + lane;  // this lane's particles of the tile: i0 + 32 k
-
+#pragma unroll
+  for (int k = 0; k < RI; ++k) {
+    const int i = t * TI + i0 + 32 * k;
+    const float *r = rec + (size_t)(i < N ? i : 0) * DP;
+#pragma unroll
+    for (int d = 0; d < D; ++d) xi[k][d] = i < N ? r[d] : VDS_PAD_COORD;
+    wi[k] = GRAD && i < N ? r[D] : 0.f;
+#pragma unroll
+    for (int a = 0; a < ACC; ++a) {
+      acc[k][a] = 0.f;
+      ks[(k * ACC + a) * NT + tid] = 0.f;
+      kc[(k * ACC + a) * NT + tid] = 0.f;
+    }
+  }
   auto fold = [&]() {
 #pragma unroll
     for (int k = 0; k < RI; ++k)
@@ -149,48 +159,13 @@ __global__ void __launch_bounds__(NT, MINB)
       }
     nf = 0;
   };
-  auto flush = [&]() {
-    fold();
-    const int seg = (int)blockIdx.x - sched_first_cta(sched_start(cur, sc), sc);
-#pragma unroll
-    for (int k = 0; k < RI; ++k)
-#pragma unroll
-      for (int a = 0; a < ACC; ++a) {
-        const int o = (k * ACC + a) * NT + tid;
-        part[(((size_t)cur * sc.maxseg + seg) * ACC + a) * TI + i0 + 32 * k] = make_float2(ks[o], -kc[o]);
-      }
-  };
-
   cp_async_wait_all();
   __syncthreads();
-  for (long long it = it0; it < it1; ++it) {
-    const int b = (int)((it - it0) & 1);
-    if (t != cur) {
-      if (cur >= 0) flush();
-      cur = t;
-#pragma unroll
-      for (int k = 0; k < RI; ++k) {
-        const int i = t * TI + i0 + 32 * k;
-        const float *r = rec + (size_t)(i < N ? i : 0) * DP;
-#pragma unroll
-        for (int d = 0; d < D; ++d) xi[k][d] = i < N ? r[d] : VDS_PAD_COORD;
-        wi[k] = GRAD && i < N ? r[D] : 0.f;
-#pragma unroll
-        for (int a = 0; a < ACC; ++a) {
-          acc[k][a] = 0.f;
-          ks[(k * ACC + a) * NT + tid] = 0.f;
-          kc[(k * ACC + a) * NT + tid] = 0.f;
-        }
-      }
-    }
-    // the next item's records arrive while this one is computed; its buffer
-    // was read last before the barrier that ended the previous item
-    int tn = t, cn = c + 1;
-    if (cn == sc.nchunk) {
-      ++tn;
-      cn = tn * CPT;
-    }
-    if (it + 1 < it1) stage(cn, b ^ 1);
+  for (int c = ca; c < cb; ++c) {
+    const int b = (c - ca) & 1;
+    // the next chunk's records arrive while this one is computed; its buffer
+    // was read last before the barrier that ended the previous chunk
+    if (c + 1 < cb) stage(c + 1, b ^ 1);
 
     const float4 *tl = tile + b * V * TJS;
     float *mj = js + (size_t)(b * W + warp) * JS::FLOATS;
@@ -291,10 +266,9 @@ __global__ void __launch_bounds__(NT, MINB)
     cp_async_wait_all();
     __syncthreads();
     // the chunk's j sums over the warps, in order; this slot buffer is written
-    // again only after the next item's barrier
+    // again only after the next chunk's barrier
     if (!diag) {
-      const long long ncol = sched_jcols(t, sc);
-      float2 *row = partj + (size_t)sched_jrow(t, sc) * ACC + (size_t)(c - (t + 1) * CPT) * TJS;
+      float2 *row = jrow + (size_t)(c - (t + 1) * CPT) * TJS;
       const float *sb = js + (size_t)b * W * JS::FLOATS;
 #pragma unroll 1
       for (int x = tid; x < TJS * ACC; x += NT) {
@@ -311,10 +285,42 @@ __global__ void __launch_bounds__(NT, MINB)
         row[(size_t)a * ncol + j] = make_float2(s, -cm);
       }
     }
-    t = tn;
-    c = cn;
   }
-  flush();
+  fold();
+#pragma unroll
+  for (int k = 0; k < RI; ++k)
+#pragma unroll
+    for (int a = 0; a < ACC; ++a) {
+      const int o = (k * ACC + a) * NT + tid;
+      ipart[(size_t)a * TI + i0 + 32 * k] = make_float2(ks[o], -kc[o]);
+    }
+}
+
+template <int D, int RI, int NT, int MINB, bool GRAD, int TJS>
+__global__ void __launch_bounds__(NT, MINB)
+    k_sym(const float *__restrict__ rec, Sched sc, int N, float2 *__restrict__ part, float2 *__restrict__ partj,
+          const ImpState *imp) {
+  constexpr int ACC = GRAD ? D : 1, TI = NT * RI, CPT = TI / TJS;
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  const long long it0 = (long long)blockIdx.x * sc.items / sc.G;
+  const long long it1 = (long long)(blockIdx.x + 1) * sc.items / sc.G;
+  if (it0 >= it1 || (imp && !imp_due(imp, GRAD))) return;  // uniform over the CTA
+  // i-tile of the first item
+  int t = 0, hi = sc.n_itiles;
+  while (hi - t > 1) {
+    const int m = (t + hi) >> 1;
+    if (sched_start(m, sc) <= it0) t = m;
+    else hi = m;
+  }
+  for (long long it = it0; it < it1; ++t) {
+    const long long s = sched_start(t, sc), e = sched_start(t + 1, sc);
+    const int ca = t * CPT + (int)(it - s), cb = t * CPT + (int)((e < it1 ? e : it1) - s);
+    const int seg = (int)blockIdx.x - sched_first_cta(s, sc);
+    sym_run<D, RI, NT, GRAD, TJS>(rec, N, t, ca, cb, sm_raw, part + ((size_t)t * sc.maxseg + seg) * ACC * TI,
+                                  partj + (size_t)sched_jrow(t, sc) * ACC, sched_jcols(t, sc));
+    it = e;
+    __syncthreads();  // the next tile's first chunk reuses the buffers
+  }
 }
 
 }  // namespace vds_pair
