@@ -55,6 +55,7 @@ struct BCommon {
   int nb, s, spring, max_iter;
   double H[8];
   double b, kBT, zeta, dt, tol, jfloor;
+  double rzeta, zeta_dt, dt_zeta;  // 1/zeta, zeta/dt (0 where dt = 0), dt/zeta
 };
 
 enum { ST_TRIAL = 0, ST_GRAD = 1, ST_FINAL = 2, ST_DONE = 3 };
@@ -235,8 +236,7 @@ struct BSymCfg {
 
 struct BUnit {
   int e, t, ca, cb;
-  int run;  // its place among the i sums
-  int pad;
+  long long run;  // its place among the i sums
 };
 // Per ensemble: first entry of its i-tiles in the table of runs, first element
 // of its j sums (in columns, times D), j-chunks; tiles < 0: not taken here.
@@ -345,40 +345,6 @@ __global__ void __launch_bounds__(32 * D)
 
 // ------------------------------------------------------ per-particle kernels
 
-__device__ __forceinline__ double bA(int j, int k) {
-  return j == k ? 2.0 : ((j - k == 1 || k - j == 1) ? -1.0 : 0.0);
-}
-__device__ __forceinline__ double bAinv(int j, int k, int nb) {
-  const int lo = (j < k ? j : k) + 1, hi = (j > k ? j : k) + 1;
-  return (double)lo * (double)(nb + 1 - hi) / (double)(nb + 1);
-}
-
-template <int D>
-__device__ __forceinline__ bool bspring(const BCommon &cm, const double (&y)[D], double &psi, double (&f)[8]) {
-  psi = 0.0;
-  bool ok = true;
-  for (int k = 0; k < cm.nb; ++k) {
-    double n2 = 0.0;
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-      if (a / cm.s == k) n2 += y[a] * y[a];
-    if (cm.spring == 0) {
-      psi += 0.5 * cm.H[k] * n2;
-      f[k] = cm.H[k];
-    } else {
-      const double x = 1.0 - n2 / cm.b;
-      if (!(x > 0.0)) {
-        ok = false;
-        f[k] = 0.0;
-      } else {
-        psi += -0.5 * cm.H[k] * cm.b * log(x);
-        f[k] = cm.H[k] / x;
-      }
-    }
-  }
-  return ok;
-}
-
 template <int D>
 __device__ __forceinline__ void write_rec(float *rec, long i, float c, const float (&y)[D]) {
   constexpr int DP = Rec<D>::DP;
@@ -469,125 +435,149 @@ __global__ void k_bprep(long total, const int *__restrict__ ens, const EParam *_
 // mode 0: density finish (w, rho_out, energy terms in contrib[3i]);
 // mode 1: gradient output g; mode 2: explicit Euler update + records;
 // mode 3: implicit round (trial: w and J terms; gradient: g -> direction).
-template <int D>
-__global__ void k_bfin(long total, const int *__restrict__ ens, const EParam *__restrict__ ep,
-                       const BState *__restrict__ st, const BCommon cm, int mode, int want_energy,
-                       const double *__restrict__ acc, float *rec, float *q, const float *__restrict__ qs,
-                       const float *dA, const float *dB, float *dir, float *__restrict__ out,
-                       double *__restrict__ contrib, int *err) {
-  constexpr int DP = Rec<D>::DP;
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const int e = ens[i];
+//
+// One thread per (particle, component), 32 particles per CTA: with one thread
+// per particle and the space dimension known only at run time, 534000 particles
+// took 221 us; 140 now, which the FP64 pipe bounds (two lanes a cycle per SM).
+template <int D, int S>
+__global__ void __launch_bounds__(32 * D)
+    k_bfin(long total, const int *__restrict__ ens, const EParam *__restrict__ ep, const BState *__restrict__ st,
+           const BCommon cm, int mode, int want_energy, const double *__restrict__ acc, float *rec, float *q,
+           const float *__restrict__ qs, const float *dA, const float *dB, float *dir, float *__restrict__ out,
+           double *__restrict__ contrib, int *err) {
+  constexpr int DP = Rec<D>::DP, NB = D / S;
+  __shared__ double sy[D][32], sd[D][32], sg[D][32], sc[D][32];
+  __shared__ float so[D][32];
+  const int p = threadIdx.x & 31, a = threadIdx.x >> 5, k = a / S, al = a - k * S;
+  const long i = (long)blockIdx.x * 32 + p;
+  const int e = i < total ? ens[i] : 0;
   const EParam &P = ep[e];
-  int phase = -1;
-  const float *dcur = nullptr, *doth = nullptr;
-  if (mode == 3) {
-    const BState s = st[e];
-    phase = s.phase;
-    dcur = s.cur ? dB : dA;
-    doth = s.cur ? dA : dB;
-    if (phase != ST_TRIAL && phase != ST_GRAD) return;
+  bool on = i < total, dens = mode == 0;
+  const float *disp = nullptr;
+  if (mode == 3 && on) {
+    const int phase = st[e].phase, cur = st[e].cur;
+    dens = phase == ST_TRIAL;
+    on = dens || phase == ST_GRAD;
+    disp = (cur != 0) == dens ? dA : dB;  // a trial's displacement is in the other buffer
   }
-  const bool dens = mode == 0 || (mode == 3 && phase == ST_TRIAL);
-  double y[D];
-  float yf[D];
+  const size_t x = (size_t)i * D + a;
+  if (on) {
+    const float d = mode == 3 ? disp[x] : 0.f;
+    sy[a][p] = (double)(mode == 3 ? qs[x] + d : q[x]);
+    sd[a][p] = (double)d;
+  }
+  __syncthreads();
+  double psi = 0.0, f = 0.0, aid = 0.0;
+  bool ok = true;
+  if (on) {
+    double n2 = 0.0;
 #pragma unroll
-  for (int d = 0; d < D; ++d) {
-    float v;
-    if (mode == 3) v = qs[(size_t)i * D + d] + (phase == ST_TRIAL ? doth : dcur)[(size_t)i * D + d];
-    else v = q[(size_t)i * D + d];
-    yf[d] = v;
-    y[d] = (double)v;
+    for (int b = 0; b < S; ++b) n2 += sy[k * S + b][p] * sy[k * S + b][p];
+    f = cm.H[k];
+    psi = 0.5 * f * n2;
+    if (cm.spring == 1) {
+      const double w = 1.0 - n2 / cm.b;
+      ok = w > 0.0;
+      psi = ok && dens && al == 0 ? -0.5 * cm.H[k] * cm.b * log(w) : 0.0;
+      f = ok ? f / w : 0.0;
+    }
+    if (mode == 3)
+#pragma unroll
+      for (int kb = 0; kb < NB; ++kb) aid += vds_pair::rouse_Ainv<NB>(k, kb) * sd[kb * S + al][p];
   }
-  double psi, fk[8];
-  const bool ok = bspring<D>(cm, y, psi, fk);
-  if (dens) {
-    const double rho = acc[(size_t)i * D];
-    if (!(rho >= 0.5 && rho <= 1e300)) vds_flag(err, VDS_ENAN);
-    rec[(size_t)i * DP + D] = (float)(1.0 / rho);
-    if (mode == 0 && out) out[i] = (float)rho;
+  // densities: energy terms; gradients: g
+  double rho = 0.0, g = 0.0, t = 0.0;
+  if (on && dens) {
+    rho = acc[(size_t)i * D];
+    if (al == 0) t = psi;
+    if (a == 0) {
+      if (!(rho >= 0.5 && rho <= 1e300)) vds_flag(err, VDS_ENAN);
+      rec[(size_t)i * DP + D] = (float)(1.0 / rho);
+      if (mode == 0 && out) out[i] = (float)rho;
+      if (want_energy || mode == 3) t += cm.kBT * (log(rho) + P.lnorm);
+    }
+    if (mode == 3) t += 0.5 * cm.zeta_dt * sd[a][p] * aid;
     if (mode == 0 && !ok && want_energy) vds_flag(err, VDS_EDOMAIN);
-    if (want_energy || mode == 3) {
-      double en = cm.kBT * (log(rho) + P.lnorm) + psi;
-      if (mode == 3) {
-        double quad = 0.0;
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-#pragma unroll
-          for (int b = 0; b < D; ++b)
-            if (a % cm.s == b % cm.s)
-              quad += (double)doth[(size_t)i * D + a] * bAinv(a / cm.s, b / cm.s, cm.nb) *
-                      (double)doth[(size_t)i * D + b];
-        en += cm.zeta / (2.0 * cm.dt) * quad;
-      }
-      contrib[3 * i] = en;
-      contrib[3 * i + 1] = ok ? 0.0 : 1.0;
-      contrib[3 * i + 2] = 0.0;
-    }
-    return;
+  } else if (on) {
+    if (!ok) vds_flag(err, VDS_EDOMAIN);
+    g = cm.kBT * (-P.sfac * acc[x]) + f * sy[a][p];
+    sg[a][p] = g;
   }
-  if (!ok) vds_flag(err, VDS_EDOMAIN);
-  double g[D];
+  sc[a][p] = t;
+  so[a][p] = ok ? 0.f : 1.f;
+  __syncthreads();
+  if (on && dens && a == 0 && (want_energy || mode == 3)) {
+    double en = 0.0;
+    float bad = 0.f;
 #pragma unroll
-  for (int a = 0; a < D; ++a) g[a] = cm.kBT * (-P.sfac * acc[(size_t)i * D + a]) + fk[a / cm.s] * y[a];
+    for (int b = 0; b < D; ++b) {
+      en += sc[b][p];
+      bad = fmaxf(bad, so[b][p]);
+    }
+    contrib[3 * i] = en;
+    contrib[3 * i + 1] = (double)bad;
+    contrib[3 * i + 2] = 0.0;
+  }
+  if (mode == 0) return;
   if (mode == 1) {
-#pragma unroll
-    for (int a = 0; a < D; ++a) out[(size_t)i * D + a] = (float)g[a];
+    if (on) out[x] = (float)g;
     return;
   }
+  double m = 0.0;  // (A g)_k: 2 on the diagonal of the Rouse matrix, -1 beside it
+  if (on && !dens) {
+    m = 2.0 * g;
+    if (k > 0) m -= sg[a - S][p];
+    if (k + 1 < NB) m -= sg[a + S][p];
+  }
+  __syncthreads();  // sc and so have been read
   if (mode == 2) {
-    float yn[D];
+    float yn = 0.f;
+    if (on) {
+      double v = 0.0;
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      const int k = a / cm.s, al = a - k * cm.s;
-      double v = 0.0, m = 0.0;
+      for (int be = 0; be < S; ++be) v += P.kappa[al * S + be] * sy[k * S + be][p];
+      yn = (float)(sy[a][p] + cm.dt * (v - m * cm.rzeta));
+      q[x] = yn;
+      rec[(size_t)i * DP + a] = P.c * yn;
+      if (a == 0)
 #pragma unroll
-      for (int b = 0; b < D; ++b) {
-        const int kb = b / cm.s, be = b - kb * cm.s;
-        if (kb == k) v += P.kappa[al * cm.s + be] * y[b];
-        if (be == al) m += bA(k, kb) * g[b];
-      }
-      yn[a] = (float)(y[a] + cm.dt * (v - m / cm.zeta));
+        for (int d = D; d < DP; ++d) rec[(size_t)i * DP + d] = 0.f;
     }
-    if (cm.spring == 1)
-      for (int k = 0; k < cm.nb; ++k) {
+    if (cm.spring == 1) {
+      so[a][p] = yn;
+      __syncthreads();
+      if (on && al == 0) {
         double n2 = 0.0;
 #pragma unroll
-        for (int a = 0; a < D; ++a)
-          if (a / cm.s == k) n2 += (double)yn[a] * yn[a];
+        for (int b = 0; b < S; ++b) n2 += (double)so[a + b][p] * so[a + b][p];
         if (!(n2 < cm.b)) vds_flag(err, VDS_EDOMAIN);
       }
-#pragma unroll
-    for (int a = 0; a < D; ++a) q[(size_t)i * D + a] = yn[a];
-    write_rec<D>(rec, i, P.c, yn);
+    }
     return;
   }
   // mode 3, new direction
-  double dec = 0.0, dmax = 0.0, ymax = 0.0;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const int k = a / cm.s, al = a - k * cm.s;
-    double ag = 0.0, aid = 0.0;
+  if (on && !dens) {
+    const double dr = sd[a][p] + cm.dt_zeta * m;
+    const double G = cm.zeta_dt * aid + g;
+    const float drf = (float)dr;
+    dir[x] = drf;
+    sc[a][p] = G * dr;
+    so[a][p] = fabsf(drf);
+  }
+  __syncthreads();
+  if (on && !dens && a == 0) {
+    double dec = 0.0, ymax = 0.0;
+    float dmax = 0.f;
 #pragma unroll
     for (int b = 0; b < D; ++b) {
-      const int kb = b / cm.s, be = b - kb * cm.s;
-      if (be == al) {
-        ag += bA(k, kb) * g[b];
-        aid += bAinv(k, kb, cm.nb) * (double)dcur[(size_t)i * D + b];
-      }
+      dec += sc[b][p];
+      dmax = fmaxf(dmax, so[b][p]);
+      ymax = fmax(ymax, fabs(sy[b][p]));
     }
-    const double dr = (double)dcur[(size_t)i * D + a] + cm.dt / cm.zeta * ag;
-    const double G = cm.zeta / cm.dt * aid + g[a];
-    const float drf = (float)dr;
-    dir[(size_t)i * D + a] = drf;
-    dec += G * dr;
-    dmax = fmax(dmax, fabs((double)drf));
-    ymax = fmax(ymax, fabs((double)yf[a]));
+    contrib[3 * i] = dec;
+    contrib[3 * i + 1] = (double)dmax;
+    contrib[3 * i + 2] = ymax;
   }
-  contrib[3 * i] = dec;
-  contrib[3 * i + 1] = dmax;
-  contrib[3 * i + 2] = ymax;
 }
 
 // One CTA per ensemble: fixed-order sums of the particles' contributions.
@@ -776,6 +766,10 @@ struct vds_batch {
   int *d_runs = nullptr;
   int2 *d_blocks = nullptr;
   float2 *ipart = nullptr, *jpart = nullptr;
+  char *sym_table = nullptr;    // holds the four tables
+  float2 *sym_work = nullptr;   // holds ipart and jpart
+  cudaStream_t side = nullptr;  // the small ensembles' pass next to the large ones'
+  cudaEvent_t fork = nullptr, join = nullptr;
   cudaGraphExec_t round_exec = nullptr;
   cudaGraph_t round_graph = nullptr;
   cudaStream_t graph_stream = nullptr;  // stream the round graph was captured for
@@ -785,18 +779,34 @@ struct vds_batch {
 namespace {
 
 template <int D, int RI, int NT>
-int b_launch_cfg(vds_ctx *c, vds_batch *b, int mode) {
-  if (!b->nord) return VDS_OK;
-  k_bpair<D, RI, NT><<<b->grid, NT, b->smem, c->stream>>>(b->rec, b->d_off, b->d_sizes, b->d_queue, b->nord,
-                                                           b->d_counter, mode, b->d_st, b->acc, c->err);
+int b_launch_cfg(vds_ctx *c, vds_batch *b, int mode, cudaStream_t st) {
+  k_bpair<D, RI, NT><<<b->grid, NT, b->smem, st>>>(b->rec, b->d_off, b->d_sizes, b->d_queue, b->nord, b->d_counter,
+                                                   mode, b->d_st, b->acc, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
+  ++c->launches;
   return VDS_OK;
 }
 
+// Both passes of a batch: the few and short items of the small ensembles on a
+// second stream (they alone left most SMs idle for 137 us of 1.6 ms), launched
+// first so that they have their SMs when the large ones' units fill the rest.
 template <int D>
 int b_launch_pair(vds_ctx *c, vds_batch *b, int mode) {
   VDS_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(unsigned), c->stream));
   VDS_TRY(vds_time_begin(c, mode == 1 ? PK_GRADIENT : PK_DENSITY));
+  const bool two = b->nord && b->nunits;
+  const cudaStream_t os = two ? b->side : c->stream;
+  if (two) {
+    VDS_CUDA_TRY(cudaEventRecord(b->fork, c->stream));
+    VDS_CUDA_TRY(cudaStreamWaitEvent(os, b->fork, 0));
+  }
+  if (b->nord) switch (b->cfg) {
+      case 0: VDS_TRY((b_launch_cfg<D, kCfgRI[0], kCfgNT[0]>(c, b, mode, os))); break;
+      case 1: VDS_TRY((b_launch_cfg<D, kCfgRI[1], kCfgNT[1]>(c, b, mode, os))); break;
+      case 2: VDS_TRY((b_launch_cfg<D, kCfgRI[2], kCfgNT[2]>(c, b, mode, os))); break;
+      default: VDS_TRY((b_launch_cfg<D, kCfgRI[3], kCfgNT[3]>(c, b, mode, os))); break;
+    }
+  if (two) VDS_CUDA_TRY(cudaEventRecord(b->join, os));
   if (b->nunits) {
     k_bsym<D><<<b->sym_grid, BSYM_NT, BSymCfg<D>::SMEM, c->stream>>>(b->rec, b->d_off, b->d_sizes, b->d_units,
                                                                      b->nunits, b->d_bens, b->d_counter + 1, mode,
@@ -807,15 +817,8 @@ int b_launch_pair(vds_ctx *c, vds_batch *b, int mode) {
     VDS_CUDA_TRY(cudaGetLastError());
     c->launches += 2;
   }
-  switch (b->cfg) {
-    case 0: VDS_TRY((b_launch_cfg<D, kCfgRI[0], kCfgNT[0]>(c, b, mode))); break;
-    case 1: VDS_TRY((b_launch_cfg<D, kCfgRI[1], kCfgNT[1]>(c, b, mode))); break;
-    case 2: VDS_TRY((b_launch_cfg<D, kCfgRI[2], kCfgNT[2]>(c, b, mode))); break;
-    default: VDS_TRY((b_launch_cfg<D, kCfgRI[3], kCfgNT[3]>(c, b, mode))); break;
-  }
-  VDS_TRY(vds_time_end(c, mode == 1 ? PK_GRADIENT : PK_DENSITY));
-  if (b->nord) ++c->launches;
-  return VDS_OK;
+  if (two) VDS_CUDA_TRY(cudaStreamWaitEvent(c->stream, b->join, 0));
+  return vds_time_end(c, mode == 1 ? PK_GRADIENT : PK_DENSITY);
 }
 
 template <int D>
@@ -829,9 +832,15 @@ int b_prep(vds_ctx *c, vds_batch *b, int mode, float *q) {
 
 template <int D>
 int b_fin(vds_ctx *c, vds_batch *b, int mode, int want_energy, float *q, float *out) {
-  k_bfin<D><<<(unsigned)((b->total + 255) / 256), 256, 0, c->stream>>>(
-      b->total, b->d_ens, b->d_ep, b->d_st, b->cm, mode, want_energy, b->acc, b->rec, q, b->qs, b->dA, b->dB,
-      b->dir, out, b->contrib, c->err);
+  const unsigned nb = (unsigned)((b->total + 31) / 32);
+  auto go = [&](auto kern) {
+    kern<<<nb, 32 * D, 0, c->stream>>>(b->total, b->d_ens, b->d_ep, b->d_st, b->cm, mode, want_energy, b->acc, b->rec,
+                                       q, b->qs, b->dA, b->dB, b->dir, out, b->contrib, c->err);
+  };
+  if constexpr (D % 2 == 0)
+    if (b->cm.s == 2) go(k_bfin<D, 2>);
+  if constexpr (D % 3 == 0)
+    if (b->cm.s == 3) go(k_bfin<D, 3>);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   return VDS_OK;
@@ -930,7 +939,7 @@ int b_setup_sym(vds_ctx *c, vds_batch *b) {
     for (int t = 0; t < ntile; ++t) {
       runs.push_back(nrun);
       for (int ca = t * C::CPT; ca < nchunk; ca += BSYM_RUN)
-        units.push_back(BUnit{e, t, ca, std::min(nchunk, ca + BSYM_RUN), nrun++, 0});
+        units.push_back(BUnit{e, t, ca, std::min(nchunk, ca + BSYM_RUN), nrun++});
     }
     runs.push_back(nrun);
     jcol += ej;
@@ -942,24 +951,32 @@ int b_setup_sym(vds_ctx *c, vds_batch *b) {
   int occ = 0;
   VDS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bsym<D>, BSYM_NT, C::SMEM));
   const long long grid = (long long)c->num_sms * (occ > 0 ? occ : 1);
-  auto put = [&](void **dst, const void *src, size_t bytes) -> cudaError_t {
-    const cudaError_t e = cudaMalloc(dst, bytes);
-    return e != cudaSuccess || !src ? e : cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-  };
-  cudaError_t ce = put((void **)&b->d_units, units.data(), units.size() * sizeof(BUnit));
-  if (ce == cudaSuccess) ce = put((void **)&b->d_bens, ens.data(), ens.size() * sizeof(BEns));
-  if (ce == cudaSuccess) ce = put((void **)&b->d_runs, runs.data(), runs.size() * sizeof(int));
-  if (ce == cudaSuccess) ce = put((void **)&b->d_blocks, blocks.data(), blocks.size() * sizeof(int2));
-  if (ce == cudaSuccess) ce = put((void **)&b->ipart, nullptr, (size_t)nrun * C::TI * D * sizeof(float2));
-  if (ce == cudaSuccess) ce = put((void **)&b->jpart, nullptr, ((size_t)jcol * D + 1) * sizeof(float2));
+  // one table, one workspace
+  const size_t bu = units.size() * sizeof(BUnit), be = ens.size() * sizeof(BEns), bb = blocks.size() * sizeof(int2),
+               br = runs.size() * sizeof(int);
+  std::vector<char> table(bu + be + bb + br);
+  memcpy(table.data(), units.data(), bu);
+  memcpy(table.data() + bu, ens.data(), be);
+  memcpy(table.data() + bu + be, blocks.data(), bb);
+  memcpy(table.data() + bu + be + bb, runs.data(), br);
+  const size_t ni = (size_t)nrun * C::TI * D, nj = (size_t)jcol * D;
+  cudaError_t ce = cudaMalloc((void **)&b->sym_work, (ni + nj) * sizeof(float2));
+  if (ce == cudaSuccess) ce = cudaMalloc((void **)&b->sym_table, table.size());
   if (ce == cudaErrorMemoryAllocation) {
     (void)cudaGetLastError();
     b->sym.assign(b->E, 0);  // all ensembles over ordered pairs
-    if (b->ipart) cudaFree(b->ipart);
-    b->ipart = nullptr;
+    if (b->sym_work) cudaFree(b->sym_work);
+    b->sym_work = nullptr;
     return VDS_OK;
   }
+  if (ce == cudaSuccess) ce = cudaMemcpy(b->sym_table, table.data(), table.size(), cudaMemcpyHostToDevice);
   VDS_CUDA_TRY(ce);
+  b->d_units = (BUnit *)b->sym_table;
+  b->d_bens = (BEns *)(b->sym_table + bu);
+  b->d_blocks = (int2 *)(b->sym_table + bu + be);
+  b->d_runs = (int *)(b->sym_table + bu + be + bb);
+  b->ipart = b->sym_work;
+  b->jpart = b->sym_work + ni;
   b->nunits = (int)units.size();
   b->nblocks = (int)blocks.size();
   b->sym_grid = (int)(grid < b->nunits ? grid : b->nunits);
@@ -1169,10 +1186,13 @@ void vds_batch_free(vds_batch *b) {
   b_drop_graph(b);
   void *ptrs[] = {b->d_off, b->d_sizes, b->d_ens, b->d_active, b->d_queue, b->d_counter, b->d_ep, b->d_st,
                   b->rec, b->qs, b->dA, b->dB, b->dir, b->dprev, b->acc, b->contrib, b->eout,
-                  b->d_units, b->d_bens, b->d_runs, b->d_blocks, b->ipart, b->jpart};
+                  b->sym_table, b->sym_work};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (b->h_active) cudaFreeHost(b->h_active);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
+  if (b->side) cudaStreamDestroy(b->side);
   delete b;
 }
 
@@ -1200,6 +1220,9 @@ int vds_batch_create(vds_ctx *c, int E, const int *sizes, int D, const vds_param
   b->cm.kBT = p->kBT;
   b->cm.zeta = p->zeta;
   b->cm.dt = p->dt;
+  b->cm.rzeta = 1.0 / p->zeta;
+  b->cm.zeta_dt = p->dt != 0.0 ? p->zeta / p->dt : 0.0;
+  b->cm.dt_zeta = p->dt / p->zeta;
   b->cm.tol = p->tol;
   b->cm.jfloor = p->jfloor;
   b->scheme = p->scheme;
@@ -1250,6 +1273,9 @@ int vds_batch_create(vds_ctx *c, int E, const int *sizes, int D, const vds_param
   A((void **)&b->contrib, sizeof(double) * 3 * tot);
   A((void **)&b->eout, sizeof(double) * E);
   if (ce == cudaSuccess) ce = cudaMallocHost((void **)&b->h_active, sizeof(int));
+  if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+  if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
   if (ce == cudaSuccess) ce = cudaMemcpy(b->d_off, b->off.data(), sizeof(long long) * E, cudaMemcpyHostToDevice);
   if (ce == cudaSuccess) ce = cudaMemcpy(b->d_sizes, sizes, sizeof(int) * E, cudaMemcpyHostToDevice);
   if (ce == cudaSuccess) ce = cudaMemcpy(b->d_ens, ens.data(), sizeof(int) * tot, cudaMemcpyHostToDevice);
