@@ -39,8 +39,11 @@ __device__ __forceinline__ void jac_pair(int a, int rnd, int Mp, int &p, int &q)
     p = rnd;
     q = Mp - 1;
   } else {
-    p = (rnd + a) % (Mp - 1);
-    q = (rnd - a + Mp - 1) % (Mp - 1);
+    // both sums lie in [0, 2 (Mp - 1)): no division on the round's critical path
+    p = rnd + a;
+    q = rnd - a + Mp - 1;
+    if (p >= Mp - 1) p -= Mp - 1;
+    if (q >= Mp - 1) q -= Mp - 1;
   }
   if (p > q) {
     const int t = p;
@@ -59,11 +62,10 @@ __device__ __forceinline__ void jac_pair(int a, int rnd, int Mp, int &p, int &q)
 // rounding), so R is orthogonal to FP64 rounding and R^T A R a similarity.
 // The (p, q) entry drops to ~1e-7 of itself instead of to zero; the next
 // sweeps take it further, at the pace of the exact rotation's convergence.
-__device__ __forceinline__ double2 jac_rot(const double *A, int M, int p, int q) {
-  if (q >= M) return make_double2(1.0, 0.0);
-  const double apq = A[(size_t)p * M + q];
+// apq, app, aqq: the pair's entries (apq 0 where there is no rotation).
+__device__ __forceinline__ double2 jac_rot(double apq, double app, double aqq) {
   if (apq == 0.0) return make_double2(1.0, 0.0);
-  const double dqp = A[(size_t)q * M + q] - A[(size_t)p * M + p];
+  const double dqp = aqq - app;
   // scale both by 2^-e, e the exponent of apq (|apq 2^-e| in [1, 2)); the
   // scale is built from its bits (e in [-1022, 1022]; outside, apq is
   // subnormal or within a factor 2 of overflow, and the pair is left alone)
@@ -114,6 +116,18 @@ __global__ void __launch_bounds__(JR_NT)
     const int tb = ta + bt;
     const int a = ta * JT + tid / JT, b = tb * JT + tid % JT;
     const bool act = a < H && b < H && a <= b;
+    // the rotations' entries first: they head the longest chain
+    double apq = 0.0, app = 0.0, aqq = 0.0;
+    if (tid < 2 * JT) {
+      const int ar = (tid < JT ? ta : tb) * JT + (tid % JT);
+      int pr, qr;
+      jac_pair(ar, rnd, Mp, pr, qr);
+      if (ar < H && qr < M) {
+        apq = A[(size_t)pr * M + qr];
+        app = A[(size_t)pr * M + pr];
+        aqq = A[(size_t)qr * M + qr];
+      }
+    }
     int p = 0, q = 0, p2 = 0, q2 = 0;
     double x00 = 0.0, x01 = 0.0, x10 = 0.0, x11 = 0.0;
     auto get = [&](int i, int j) -> double { return (i < M && j < M) ? A[(size_t)i * M + j] : 0.0; };
@@ -125,16 +139,7 @@ __global__ void __launch_bounds__(JR_NT)
       x10 = get(q, p2);
       x11 = get(q, q2);
     }
-    if (tid < 2 * JT) {
-      const int ar = (tid < JT ? ta : tb) * JT + (tid % JT);
-      double2 r = make_double2(1.0, 0.0);
-      if (ar < H) {
-        int pr, qr;
-        jac_pair(ar, rnd, Mp, pr, qr);
-        r = jac_rot(A, M, pr, qr);
-      }
-      rot[tid] = r;
-    }
+    if (tid < 2 * JT) rot[tid] = jac_rot(apq, app, aqq);
     __syncthreads();
     if (!act) return;
     const double2 ra = rot[tid / JT], rb = rot[JT + tid % JT];
@@ -166,6 +171,12 @@ __global__ void __launch_bounds__(JR_NT)
     int p2 = 0, q2 = 0;
     double vp[VR], vq[VR];
     if (b < H) jac_pair(b, rnd, Mp, p2, q2);
+    double apq = 0.0, app = 0.0, aqq = 0.0;
+    if (tid < JT && b < H && q2 < M) {  // there b is the pair of rotation tid
+      apq = A[(size_t)p2 * M + q2];
+      app = A[(size_t)p2 * M + p2];
+      aqq = A[(size_t)q2 * M + q2];
+    }
 #pragma unroll
     for (int k = 0; k < VR; ++k) {
       const int i = ti * JV_ROWS + tid / JT + k * (JR_NT / JT);
@@ -173,16 +184,7 @@ __global__ void __launch_bounds__(JR_NT)
       vp[k] = (ok && p2 < M) ? V[(size_t)i * M + p2] : 0.0;
       vq[k] = (ok && q2 < M) ? V[(size_t)i * M + q2] : 0.0;
     }
-    if (tid < JT) {
-      const int br = tb * JT + tid;
-      double2 r = make_double2(1.0, 0.0);
-      if (br < H) {
-        int pr, qr;
-        jac_pair(br, rnd, Mp, pr, qr);
-        r = jac_rot(A, M, pr, qr);
-      }
-      rot[tid] = r;
-    }
+    if (tid < JT) rot[tid] = jac_rot(apq, app, aqq);
     __syncthreads();
     if (b >= H) return;
     const double2 rb = rot[tid % JT];
@@ -268,20 +270,23 @@ __global__ void __launch_bounds__(1024)
     k_eig_sort(const double *__restrict__ A, const double *__restrict__ V, int M, double energy,
                int r_max, int r_fixed, double *lam_sorted, int *order, double *W, double *scal) {
   __shared__ int r_sh;
+  __shared__ double diag[2048], sorted[2048];  // M <= 2048; from global memory 322 us at M = 600
+  for (int i = threadIdx.x; i < M; i += blockDim.x) diag[i] = A[(size_t)i * M + i];
+  __syncthreads();
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    const double li = A[(size_t)i * M + i];
+    const double li = diag[i];
     int rank = 0;
     for (int j = 0; j < M; ++j) {
-      const double lj = A[(size_t)j * M + j];
+      const double lj = diag[j];
       rank += (lj > li) || (lj == li && j < i);
     }
     order[rank] = i;
-    lam_sorted[rank] = li;
+    lam_sorted[rank] = sorted[rank] = li;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double tot = 0.0;
-    for (int k = 0; k < M; ++k) tot += lam_sorted[k];
+    for (int k = 0; k < M; ++k) tot += sorted[k];
     int r;
     if (r_fixed > 0) {
       r = r_fixed < M ? r_fixed : M;
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(1024)
       r = M;
       double cum = 0.0;
       for (int k = 0; k < M; ++k) {
-        cum += lam_sorted[k];
+        cum += sorted[k];
         if (cum >= energy * tot) {
           r = k + 1;
           break;
@@ -299,7 +304,7 @@ __global__ void __launch_bounds__(1024)
     }
     // modes whose eigenvalue is not resolved in FP64 cannot be normalised
     int rp = 0;
-    while (rp < r && lam_sorted[rp] > 1e-13 * lam_sorted[0] && lam_sorted[rp] > 0.0) ++rp;
+    while (rp < r && sorted[rp] > 1e-13 * sorted[0] && sorted[rp] > 0.0) ++rp;
     scal[SC_AUX + 2] = (double)r;
     scal[SC_AUX + 3] = (double)rp;
     r_sh = rp;
@@ -308,45 +313,58 @@ __global__ void __launch_bounds__(1024)
   const int r = r_sh;
   for (int idx = threadIdx.x; idx < M * 64; idx += blockDim.x) {
     const int m = idx / 64, t = idx - (idx / 64) * 64;
-    W[idx] = t < r ? V[(size_t)m * M + order[t]] / sqrt(lam_sorted[t]) : 0.0;
+    W[idx] = t < r ? V[(size_t)m * M + order[t]] / sqrt(sorted[t]) : 0.0;
   }
 }
 
 // ---------------------------------------------------------------- basis
 
-constexpr int BT = 16;  // basis columns per CTA
-constexpr int BM = 128; // W rows staged per step
+constexpr int BM = 128;  // W rows staged per step
 
-// Phi[row, t] = sum_m X[row + m Ns] W[m, t]  (FP64 accumulation)
+// A W_r for a tile of BT columns (16, or 8 where the rank is at most 8), one
+// row per thread.  Every product x W is FP32 x FP64 and the sum FP64 in
+// effect: W in two FP32 parts, the product's rounding by a fused multiply-add,
+// the sum's by two-sum, eleven FP32 operations at 64 times the FP64 pipe's
+// rate.  196608 x 600, r = 6: 3.9 ms in FP64 on 16 columns.
+template <int BT>
 __global__ void __launch_bounds__(256)
     k_basis(const float *__restrict__ X, long Ns, int M, const double *__restrict__ W, int r, int ld,
             float *__restrict__ phi) {
-  __shared__ double Ws[BM][BT];
+  __shared__ float2 Ws[BM][BT];
   const long row = (long)blockIdx.x * 256 + threadIdx.x;
   const int t0 = blockIdx.y * BT;
-  double acc[BT];
+  float hi[BT], lo[BT];
 #pragma unroll
-  for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+  for (int t = 0; t < BT; ++t) hi[t] = lo[t] = 0.f;
   for (int m0 = 0; m0 < M; m0 += BM) {
     __syncthreads();
     for (int e = threadIdx.x; e < BM * BT; e += 256) {
       const int mm = e / BT, t = e - (e / BT) * BT;
-      Ws[mm][t] = (m0 + mm < M) ? W[(size_t)(m0 + mm) * 64 + t0 + t] : 0.0;
+      const double w = (m0 + mm < M) ? W[(size_t)(m0 + mm) * 64 + t0 + t] : 0.0;
+      const float wh = (float)w;
+      Ws[mm][t] = make_float2(wh, (float)(w - (double)wh));
     }
     __syncthreads();
     if (row < Ns) {
       const int mend = min(BM, M - m0);
+#pragma unroll 4
       for (int mm = 0; mm < mend; ++mm) {
-        const double x = (double)X[row + (long)(m0 + mm) * Ns];
+        const float x = X[row + (long)(m0 + mm) * Ns];
 #pragma unroll
-        for (int t = 0; t < BT; ++t) acc[t] = fma(x, Ws[mm][t], acc[t]);
+        for (int t = 0; t < BT; ++t) {
+          const float2 w = Ws[mm][t];
+          const float p = x * w.x, e = fmaf(x, w.x, -p);
+          const float s = hi[t] + p, b = s - hi[t];
+          lo[t] += ((hi[t] - (s - b)) + (p - b)) + fmaf(x, w.y, e);
+          hi[t] = s;
+        }
       }
     }
   }
   if (row < Ns) {
 #pragma unroll
     for (int t = 0; t < BT; ++t)
-      if (t0 + t < ld) phi[row * ld + t0 + t] = (t0 + t < r) ? (float)acc[t] : 0.f;
+      if (t0 + t < ld) phi[row * ld + t0 + t] = (t0 + t < r) ? (float)((double)hi[t] + (double)lo[t]) : 0.f;
   }
 }
 
@@ -811,31 +829,37 @@ int pod_build(vds_ctx *c, const float *X, long Ns, int M, int s, double energy, 
   const unsigned nblk_round = (unsigned)(nAt + nVt);
   int offblk = (int)((MM + 255) / 256);
   if (offblk > 256) offblk = 256;
-  // One sweep (Mpe - 1 rounds, one launch each) is captured as a CUDA graph
-  // per starting buffer pair (the buffers swap once per round).
-  struct SweepGraphs {
-    cudaGraphExec_t g[2] = {nullptr, nullptr};
-    ~SweepGraphs() {
-      for (cudaGraphExec_t x : g)
-        if (x) cudaGraphExecDestroy(x);
+  // One sweep (Mpe - 1 rounds, one launch each; the buffers swap every round)
+  // is captured as a CUDA graph.  Mpe - 1 is odd: a copy at its end brings
+  // the matrices back to the buffers it starts from, so that one graph serves
+  // every sweep (capturing and instantiating 600 nodes takes the host 2 ms).
+  struct SweepGraph {
+    cudaGraphExec_t g = nullptr;
+    ~SweepGraph() {
+      if (g) cudaGraphExecDestroy(g);
     }
   } sg;
   double *Ab[2] = {A0, A1}, *Vb[2] = {V0, V1};
-  auto capture = [&](int par) -> int {
+  auto capture = [&]() -> int {
     cudaStream_t cap;
     VDS_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-    int cur = par;
+    int cur = 0;
     for (int rnd = 0; rnd < Mpe - 1 && e == cudaSuccess; ++rnd) {
       k_jacobi_round<<<nblk_round, JR_NT, 0, cap>>>(Ab[cur], Ab[cur ^ 1], Vb[cur], Vb[cur ^ 1], M, Mpe, rnd,
                                                     nT, nAt);
       e = cudaGetLastError();
       cur ^= 1;
     }
+    if (cur) {
+      const size_t bytes = (size_t)MM * sizeof(double);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(Ab[0], Ab[1], bytes, cudaMemcpyDeviceToDevice, cap);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(Vb[0], Vb[1], bytes, cudaMemcpyDeviceToDevice, cap);
+    }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
     cudaStreamDestroy(cap);
-    if (e == cudaSuccess && e2 == cudaSuccess) e = cudaGraphInstantiate(&sg.g[par], graph, 0);
+    if (e == cudaSuccess && e2 == cudaSuccess) e = cudaGraphInstantiate(&sg.g, graph, 0);
     if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess || e2 != cudaSuccess) {
       vds_last_cuda_error(e != cudaSuccess ? e : e2);
@@ -843,15 +867,13 @@ int pod_build(vds_ctx *c, const float *X, long Ns, int M, int s, double energy, 
     }
     return VDS_OK;
   };
-  int par = 0;  // buffers holding the current A, V
   int sweeps = 0;
   double prev_off = -1.0;
   for (int sweep = 0; sweep < 40; ++sweep) {
-    if (!sg.g[par]) VDS_TRY(capture(par));
-    VDS_CUDA_TRY(cudaGraphLaunch(sg.g[par], c->stream));
+    if (!sg.g) VDS_TRY(capture());
+    VDS_CUDA_TRY(cudaGraphLaunch(sg.g, c->stream));
     c->launches += Mpe - 1;
-    if ((Mpe - 1) % 2 == 1) par ^= 1;
-    k_offnorm<<<offblk, 256, 0, c->stream>>>(Ab[par], M, (double *)c->red.ptr, c->ticket + TK_MISC, c->scal);
+    k_offnorm<<<offblk, 256, 0, c->stream>>>(Ab[0], M, (double *)c->red.ptr, c->ticket + TK_MISC, c->scal);
     VDS_CUDA_TRY(cudaGetLastError());
     ++c->launches;
     VDS_CUDA_TRY(cudaMemcpyAsync(c->h_scal, c->scal, SC_COUNT * sizeof(double), cudaMemcpyDeviceToHost,
@@ -866,8 +888,6 @@ int pod_build(vds_ctx *c, const float *X, long Ns, int M, int s, double energy, 
     if (off <= 1e-22 * tot || (prev_off >= 0.0 && off >= prev_off)) break;
     prev_off = off;
   }
-  A0 = Ab[par];
-  V0 = Vb[par];
 
   // 3. sort, rank rule, W = V_r Lambda_r^-1/2
   k_eig_sort<<<1, 1024, 0, c->stream>>>(A0, V0, M, energy, r_max, r_fixed, lam_s, order, W, c->scal);
@@ -906,8 +926,9 @@ int pod_build(vds_ctx *c, const float *X, long Ns, int M, int s, double energy, 
     }
     // 4. basis
     if ((st = vds_time_begin(c, PK_BASIS)) != VDS_OK) break;
-    k_basis<<<dim3((unsigned)((Ns + 255) / 256), (ld + BT - 1) / BT), 256, 0, c->stream>>>(X, Ns, M, W, r,
-                                                                                         ld, b->phi);
+    const unsigned rows = (unsigned)((Ns + 255) / 256);
+    if (ld <= 8) k_basis<8><<<rows, 256, 0, c->stream>>>(X, Ns, M, W, r, ld, b->phi);
+    else k_basis<16><<<dim3(rows, (ld + 15) / 16), 256, 0, c->stream>>>(X, Ns, M, W, r, ld, b->phi);
     if (cudaGetLastError() != cudaSuccess) {
       st = VDS_ECUDA;
       break;
