@@ -272,83 +272,96 @@ __global__ void k_input(const float *__restrict__ x, const int *__restrict__ row
   if (a0t) a0t[(size_t)k * ldt + m] = b;
 }
 
-// dS = (2/M)(s + eps/sigma) (first D columns), padded BF16 copies; loss terms
-__global__ void k_dsm_out(const float *__restrict__ S, int ldS, const float *__restrict__ eps, float sigma, int M,
-                          int D, float *__restrict__ dSf, int Op, bf16 *__restrict__ dSb, int ldb,
-                          bf16 *__restrict__ dSt, int ldt, double *__restrict__ lossp) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  if (m < M) {
-    for (int k = 0; k < ldb; ++k) {
-      float g = 0.f;
-      if (k < D) {
-        const float r = S[(size_t)m * ldS + k] + eps[(size_t)m * D + k] / sigma;
-        l += (double)r * r;
-        g = 2.f * r / (float)M;
-      }
-      if (k < Op) {
-        dSf[(size_t)m * Op + k] = g;
-        dSt[(size_t)k * ldt + m] = __float2bfloat16_rn(g);
-      }
-      dSb[(size_t)m * ldb + k] = __float2bfloat16_rn(g);
-    }
-  }
+// Output layer of a training step: residual r = s + eps/sigma (denoising) or
+// s - t, t = target[rows[m]] (or target[m]) (FIT), dS = (2/M) r in the first D
+// columns, its padded BF16 copies (row-major and transposed) and the rows'
+// loss terms.  64 rows x 64 columns per CTA, a thread per element and the
+// transposed copy through shared memory: one thread per row with all its
+// columns took 24 us at M = 8192.
+constexpr int OUT_ROWS = 64;
+template <bool FIT>
+__global__ void __launch_bounds__(256)
+    k_out(const float *__restrict__ S, int ldS, const float *__restrict__ ref, const int *__restrict__ rows,
+          float sigma, int M, int D, float *__restrict__ dSf, int Op, bf16 *__restrict__ dSb, bf16 *__restrict__ dSt,
+          int ldt, double *__restrict__ lossp) {
+  constexpr int LDB = 64;  // columns of dSb
+  __shared__ bf16 tr[16][OUT_ROWS + 2];  // Op <= 16
   __shared__ double sh[256];
-  sh[threadIdx.x] = l;
+  const int base = blockIdx.x * OUT_ROWS, tid = threadIdx.x;
+  double l = 0.0;
+#pragma unroll 4
+  for (int e = tid; e < OUT_ROWS * LDB; e += 256) {
+    const int ml = e / LDB, k = e % LDB, m = base + ml;
+    if (m >= M) break;
+    float g = 0.f;
+    if (k < D) {
+      const size_t x = (size_t)(FIT && rows ? rows[m] : m) * D + k;
+      const float r = FIT ? S[(size_t)m * ldS + k] - ref[x] : S[(size_t)m * ldS + k] + ref[x] / sigma;
+      l += (double)r * r;
+      g = 2.f * r / (float)M;
+    }
+    const bf16 gb = __float2bfloat16_rn(g);
+    if (k < Op) {
+      dSf[(size_t)m * Op + k] = g;
+      tr[k][ml] = gb;
+    }
+    dSb[(size_t)m * LDB + k] = gb;
+  }
+  sh[tid] = l;
   __syncthreads();
+  for (int e = tid; e < Op * OUT_ROWS; e += 256) {
+    const int k = e / OUT_ROWS, ml = e % OUT_ROWS;
+    if (base + ml < M) dSt[(size_t)k * ldt + base + ml] = tr[k][ml];
+  }
   for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    if (tid < o) sh[tid] += sh[tid + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) lossp[blockIdx.x] = sh[0];
+  if (tid == 0) lossp[blockIdx.x] = sh[0];
 }
 
-// regression: dS = (2/M)(s - t), t = target[rows[m]] (or target[m])
-__global__ void k_fit_out(const float *__restrict__ S, int ldS, const float *__restrict__ target,
-                          const int *__restrict__ rows, int M, int D, float *__restrict__ dSf, int Op,
-                          bf16 *__restrict__ dSb, int ldb, bf16 *__restrict__ dSt, int ldt,
-                          double *__restrict__ lossp) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  if (m < M) {
-    const size_t tr = (size_t)(rows ? rows[m] : m) * D;
-    for (int k = 0; k < ldb; ++k) {
-      float g = 0.f;
-      if (k < D) {
-        const float r = S[(size_t)m * ldS + k] - target[tr + k];
-        l += (double)r * r;
-        g = 2.f * r / (float)M;
-      }
-      if (k < Op) {
-        dSf[(size_t)m * Op + k] = g;
-        dSt[(size_t)k * ldt + m] = __float2bfloat16_rn(g);
-      }
-      dSb[(size_t)m * ldb + k] = __float2bfloat16_rn(g);
-    }
-  }
-  __shared__ double sh[256];
-  sh[threadIdx.x] = l;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) lossp[blockIdx.x] = sh[0];
+// Column sums of an M x n FP32 matrix in a fixed order -> out[n]: 32 columns x
+// a chunk of rows per CTA (coalesced; one CTA per column read 4 of every 32
+// bytes and took 16 us at 8192 x 256), the last CTA of a column tile adds the
+// chunks' sums.  Sums are carried as FP32 pairs (two-sum, 48 bits).
+constexpr int CS_CHUNKS = 16;
+__device__ __forceinline__ void cs_add(float2 &a, float x, float y) {
+  const float t = a.x + x, b = t - a.x;
+  a.y += ((a.x - (t - b)) + (x - b)) + y;
+  a.x = t;
 }
-
-// column sums of an M x n FP32 matrix in a fixed order -> out[n]
-__global__ void k_colsum(const float *__restrict__ X, int M, int n, int ld, float *__restrict__ out) {
-  const int col = blockIdx.x;
-  double a = 0.0;
-  for (int m = threadIdx.x; m < M; m += blockDim.x) a += X[(size_t)m * ld + col];
-  __shared__ double sh[512];
-  sh[threadIdx.x] = a;
+__global__ void __launch_bounds__(256)
+    k_colsum(const float *__restrict__ X, int M, int n, int ld, float2 *__restrict__ part, unsigned *ticket,
+             float *__restrict__ out) {
+  __shared__ float2 sh[8][32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, col = blockIdx.x * 32 + lane;
+  const int per = (M + gridDim.y - 1) / gridDim.y;
+  const int m0 = blockIdx.y * per, m1 = min(M, m0 + per);
+  float2 a = make_float2(0.f, 0.f);
+  if (col < n)
+#pragma unroll 8
+    for (int m = m0 + w; m < m1; m += 8) cs_add(a, X[(size_t)m * ld + col], 0.f);
+  sh[w][lane] = a;
   __syncthreads();
-  for (int o = 256; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+  if (w) return;
+  for (int k = 1; k < 8; ++k) cs_add(a, sh[k][lane].x, sh[k][lane].y);
+  if (col < n) part[(size_t)blockIdx.y * n + col] = a;
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) last = atomicAdd(ticket + blockIdx.x, 1u) == gridDim.y - 1;
+  __syncwarp();
+  if (!last) return;
+  __threadfence();
+  if (col < n) {
+    float2 t = make_float2(0.f, 0.f);
+    for (unsigned k = 0; k < gridDim.y; ++k) {
+      const float2 v = __ldcg(part + (size_t)k * n + col);
+      cs_add(t, v.x, v.y);
+    }
+    out[col] = (float)((double)t.x + (double)t.y);
   }
-  if (threadIdx.x == 0 && col < n) out[col] = (float)sh[0];
+  if (lane == 0) ticket[blockIdx.x] = 0u;
 }
 
 // out[i] = sum over splits of part[s * stride + i]
@@ -940,7 +953,7 @@ int ensure_acts(vds_score *s, int M) {
   A((void **)&s->sf, sizeof(float) * Mc * s->Op);
   A((void **)&s->dsf, sizeof(float) * Mc * s->Op);
   A((void **)&s->part, sizeof(float) * 64 * W * W);
-  A((void **)&s->lossp, sizeof(double) * (Mc / 256 + 1));
+  A((void **)&s->lossp, sizeof(double) * (Mc / OUT_ROWS + 1));
   if (ce != cudaSuccess) {
     vds_last_cuda_error(ce);
     free_acts(s);
@@ -995,13 +1008,13 @@ int loss_grad(vds_ctx *c, vds_score *s, const float *x, const int *rows, const f
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   VDS_TRY(forward(c, s, M, true, s->sf, s->Op, s->Op));
-  const int nb = (M + 255) / 256;
+  const int nb = (M + OUT_ROWS - 1) / OUT_ROWS;
   if (target)
-    k_fit_out<<<nb, 256, 0, c->stream>>>(s->sf, s->Op, target, rows, M, s->D, s->dsf, s->Op, s->dsb, 64, s->dst,
-                                         Mc, s->lossp);
+    k_out<true><<<nb, 256, 0, c->stream>>>(s->sf, s->Op, target, rows, 1.f, M, s->D, s->dsf, s->Op, s->dsb, s->dst,
+                                           Mc, s->lossp);
   else
-    k_dsm_out<<<nb, 256, 0, c->stream>>>(s->sf, s->Op, eps, (float)sigma, M, s->D, s->dsf, s->Op, s->dsb, 64,
-                                         s->dst, Mc, s->lossp);
+    k_out<false><<<nb, 256, 0, c->stream>>>(s->sf, s->Op, eps, nullptr, (float)sigma, M, s->D, s->dsf, s->Op, s->dsb,
+                                            s->dst, Mc, s->lossp);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   // split-K over the batch for the weight gradients
@@ -1018,7 +1031,9 @@ int loss_grad(vds_ctx *c, vds_score *s, const float *x, const int *rows, const f
     return VDS_OK;
   };
   auto bgrad = [&](const float *X, int n, int ld, float *dst) -> int {
-    k_colsum<<<n, 512, 0, c->stream>>>(X, M, n, ld, dst);
+    // (the split-K scratch is free between the weight gradients)
+    k_colsum<<<dim3((unsigned)(n + 31) / 32, CS_CHUNKS), 256, 0, c->stream>>>(X, M, n, ld, (float2 *)s->part,
+                                                                             c->ticket + TK_COLSUM, dst);
     VDS_CUDA_TRY(cudaGetLastError());
     ++c->launches;
     return VDS_OK;

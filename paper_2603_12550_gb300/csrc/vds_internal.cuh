@@ -238,4 +238,4 @@ int vds_sync_status(vds_ctx *c);  // synchronise the stream, read+clear err
 // Scalar slots in ctx->scal
 enum { SC_E = 0, SC_DEC = 1, SC_DMAX = 2, SC_YMAX = 3, SC_H = 4, SC_AUX = 5, SC_COUNT = 320 };
 // Ticket slots
-enum { TK_DENS = 0, TK_GRAD = 1, TK_STRESS = 2, TK_MISC = 3, TK_COUNT = 16 };
+enum { TK_DENS = 0, TK_GRAD = 1, TK_STRESS = 2, TK_MISC = 3, TK_COLSUM = 8 /* .. 15 */, TK_COUNT = 16 };
