@@ -192,7 +192,10 @@ extern "C" int vds_convect(vds_ctx *c, const float *q_in, float *q_out, int nx, 
   } else {
     const float cx = (float)(dt / dx[0]), cy = (float)(dt / dx[1]), cz = (float)(dt / dx[2]);
     if (wide) {
-      // block of nodes: double the shortest axis that has nodes left
+      // block of nodes: double the shortest axis that has nodes left; small
+      // fields take smaller blocks (a node per warp at least) to use every SM
+      int most = CT_NODES;
+      while (most > CT_NT / 32 && G / most * chunks < 2 * c->num_sms) most /= 2;
       CvTile T = {0, 0, 0, 0, 0, 0};
       for (;;) {
         int *const l[3] = {&T.lx, &T.ly, &T.lz};
@@ -200,7 +203,7 @@ extern "C" int vds_convect(vds_ctx *c, const float *q_in, float *q_out, int nx, 
         int best = -1;
         for (int a = 0; a < 3; ++a)
           if ((1 << *l[a]) < n[a] && (best < 0 || *l[a] < *l[best])) best = a;
-        if (best < 0 || (2 << (T.lx + T.ly + T.lz)) > CT_NODES) break;
+        if (best < 0 || (2 << (T.lx + T.ly + T.lz)) > most) break;
         ++*l[best];
       }
       T.bx = (nx + (1 << T.lx) - 1) >> T.lx;
