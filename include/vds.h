@@ -136,8 +136,8 @@ VDS_API int vds_stress(vds_ctx *ctx, const float *q, int N, int D, const vds_par
  * the query points to be the particles themselves: f(q_I) = rho_I (1/N)
  * (2 pi h^2)^(-D/2)).  q: device N x D, y: device M x D, f: device M (FP32);
  * p->nb, p->s give D.  One query-particle pair pass (query points as its
- * rows, counted as a density pass by vds_timing) with FP64 sums across
- * particle tiles.  Asynchronous on the context stream.  VDS_EARG for a NULL
+ * rows, counted as a density pass by vds_timing) with sums across
+ * particle tiles compensated in FP32 pairs.  Asynchronous on the context stream.  VDS_EARG for a NULL
  * pointer, N < 1, M < 1 or invalid parameters. */
 VDS_API int vds_density_at(vds_ctx *ctx, const float *q, int N, int D, const vds_params *p,
                            const float *y, int M, float *f);

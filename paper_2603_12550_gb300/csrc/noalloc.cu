@@ -15,12 +15,13 @@
 // synchronises its stream before returning, on success and on every error
 // return, so calls made one after another from one thread do not overlap.
 //
-// Pass shapes follow vds_energy_grad's choice (small clouds take the
-// 128-thread, 64-record shape; mid-size clouds 64-record j-chunks when their
-// partial sums fit), except that a stream-K grid whose partial sums would not
-// fit the fixed buffer is cut down until they do: at N near
-// VDS_NOALLOC_MAX_N the gradient pass runs on fewer CTAs than the context
-// path (about a quarter of the SMs at D = 9), so it is slower there.
+// The passes are the ordered ones (every row against all particles), whose
+// scratch fits the fixed buffer; vds_energy_grad takes unordered pairs, and one
+// launch for small clouds, and is faster.  Small clouds take the 128-thread,
+// 64-record shape, mid-size clouds 64-record j-chunks when their partial sums
+// fit; a stream-K grid whose partial sums would not fit the fixed buffer is cut
+// down until they do: at N near VDS_NOALLOC_MAX_N the gradient pass runs on
+// about a quarter of the SMs at D = 9.
 #include <mutex>
 
 #include "pair_impl.cuh"

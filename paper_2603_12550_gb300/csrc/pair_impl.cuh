@@ -17,7 +17,8 @@
 // (cp.async.bulk + mbarrier transaction counts) issued by one thread.  All
 // threads read the same record at a time (shared-memory broadcast).  Inside a
 // j-tile sums are plain FP32; across tiles they are Kahan-compensated; across
-// CTAs they are combined in FP64 by the epilogue in a fixed order.
+// CTAs they are left as FP32 (sum, rest) pairs, which the epilogue adds by
+// two-sums in a fixed order.
 #include <math.h>
 
 #include "pair.cuh"

@@ -213,8 +213,8 @@ struct vds_ctx {
   DevBuf rec;      // records (N_pad x DP floats)
   DevBuf rec2;     // the next step's records while a small cloud's pass reads rec
   DevBuf recq;     // records of query points (vds_density_at)
-  DevBuf part;     // pair-pass partial sums (FP64)
-  DevBuf partj;    // j-side partial sums of the symmetric passes (FP64)
+  DevBuf part;     // pair-pass partial sums (FP32 sum and rest)
+  DevBuf partj;    // j-side partial sums of the symmetric passes (FP32 sum and rest)
   DevBuf red;      // block partials of reductions (FP64)
   DevBuf vecs;     // minimiser vectors / scratch (FP32)
   DevBuf imp;      // minimiser state and iteration counts
