@@ -487,7 +487,8 @@ int launch_pass(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci, const I
 // CTAs of 128 threads per SM (MINB: the register budget) and threads per CTA
 // on GB300: the most particles per lane whose warps still fill the schedulers.
 // Gradient, N = 65536, D = 9: RI = 6 at three CTAs 2.81 ms, 5 at three 2.95,
-// 4 at four 3.18, 8 at two 3.20 (k_pair 3.86).  D = 6: 8 at three 2.10, 6 at
+// 4 at four 3.18, 8 at two 3.20 (k_pair 3.86; with the folds of sym_run every
+// 128 records, every 64 the first takes 2.93 in the bench).  D = 6: 8 at three 2.10, 6 at
 // four 2.12.  Density, D = 9: 10 at three 1.36, 8 at four 1.49, 12 at two 1.42
 // (k_pair 2.46).
 template <int D, bool GRAD>
