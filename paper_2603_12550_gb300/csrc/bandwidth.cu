@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(BrCfg<D>::NT, BrCfg<D>::MINB)
   };
   unsigned long long total = 0ull;
   // a pair of the screen's bracket: its key decides
-  auto judge = [&](unsigned key, bool on) {
+  auto sort_in = [&](unsigned key, bool on) {
     total += on && key < lo;
     const bool in = on && key - lo <= span;
     const unsigned m = __ballot_sync(0xffffffffu, in);
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(BrCfg<D>::NT, BrCfg<D>::MINB)
       while (__any_sync(0xffffffffu, w & 0xffu)) {  // nearly always one pair per entry
         const bool on = (w & 0xffu) != 0u;
         const int i = t * C::TI + (int)(w >> 16) + (__ffs(w & 0xffu) - 1) * NT;
-        judge(on ? pair_key<D>(q, i, c * TJB + (int)(w >> 8 & 0xffu)) : 0u, on);
+        sort_in(on ? pair_key<D>(q, i, c * TJB + (int)(w >> 8 & 0xffu)) : 0u, on);
         w &= w - 1u;
         if (!on) w = 0u;
       }
