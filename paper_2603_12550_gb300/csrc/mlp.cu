@@ -323,7 +323,9 @@ __global__ void __launch_bounds__(256)
 // Column sums of an M x n FP32 matrix in a fixed order -> out[n]: 32 columns x
 // a chunk of rows per CTA (coalesced; one CTA per column read 4 of every 32
 // bytes and took 16 us at 8192 x 256), the last CTA of a column tile adds the
-// chunks' sums.  Sums are carried as FP32 pairs (two-sum, 48 bits).
+// chunks' sums.  Sums are carried as FP32 pairs (two-sum, 48 bits); a column
+// whose FP32 sum leaves the finite range is added again in FP64, since a
+// two-sum makes NaN of an infinity.
 constexpr int CS_CHUNKS = 16;
 __device__ __forceinline__ void cs_add(float2 &a, float x, float y) {
   const float t = a.x + x, b = t - a.x;
@@ -359,7 +361,12 @@ __global__ void __launch_bounds__(256)
       const float2 v = __ldcg(part + (size_t)k * n + col);
       cs_add(t, v.x, v.y);
     }
-    out[col] = (float)((double)t.x + (double)t.y);
+    double s = (double)t.x + (double)t.y;
+    if (!(fabs(s) <= 3.0e38)) {
+      s = 0.0;
+      for (int m = 0; m < M; ++m) s += (double)X[(size_t)m * ld + col];
+    }
+    out[col] = (float)s;
   }
   if (lane == 0) ticket[blockIdx.x] = 0u;
 }
