@@ -17,7 +17,7 @@
  * counter; an item covers all j of its ensemble, so every particle's sums are
  * formed by one CTA in a fixed order and the results do not depend on the
  * schedule.  Ensembles of 2048 particles and more are taken over unordered
- * pairs instead, in units of their own (an i-tile against up to 1024 later
+ * pairs instead, in units of their own (an i-tile against 256 to 1024 later
  * particles) whose sums have their own places and are added in a fixed order;
  * the queue lists every ensemble's items all the same.
  */

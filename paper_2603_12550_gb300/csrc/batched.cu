@@ -2,7 +2,7 @@
 // together (include/vds_batch.h).
 //
 // Persistent pair kernels per pass.  Ensembles of BSYM_MIN_N particles and more
-// go over unordered pairs (k_bsym): units of one i-tile against up to BSYM_RUN
+// go over unordered pairs (k_bsym): units of one i-tile against up to 32
 // j-chunks, in longest-processing-time order from an atomic counter, each
 // leaving its sums in its own place; k_bgather adds a particle's in a fixed
 // order.  The units of an ensemble depend on its size alone.  Smaller ones go
@@ -224,8 +224,15 @@ __global__ void __launch_bounds__(NT)
 // tiles of 1024 is three tile pairs' work where the ordered form has four.
 constexpr int BSYM_MIN_N = 2048;
 constexpr int BSYM_TJS = 32, BSYM_NT = 128;
-constexpr int BSYM_RUN = 32;                           // j-chunks per unit
 constexpr long long BSYM_MAX_FLOAT2 = (long long)1 << 29;  // workspace: 4 GiB
+// j-chunks per unit: a sixteenth of the ensemble, 8 to 32.  The longest unit sets
+// the time of a batch that does not fill the GPU, and long units its last round;
+// shorter ones cost more tile loads and sums.  They follow the ensemble's size
+// alone, as the sum of an i-tile is cut at them: the same bits in every batch.
+// Energy and gradient of 1 / 32 / 96 ensembles of 2048 particles, D = 9: ordered
+// items 0.234 / 0.356 / 0.874 ms, units of 32 chunks 0.376 / 0.579 / 0.867, these
+// 0.137 / 0.320 / 0.744; 16 of 6144, D = 8: 1.20 / 0.72 / 0.76.
+constexpr int bsym_run(int nchunk) { return nchunk < 128 ? 8 : nchunk > 512 ? 32 : nchunk / 16; }
 
 template <int D>
 struct BSymCfg {
@@ -930,16 +937,17 @@ int b_setup_sym(vds_ctx *c, vds_batch *b) {
     if (N < BSYM_MIN_N) continue;
     const int nchunk = (N + BSYM_TJS - 1) / BSYM_TJS, ntile = (N + C::TI - 1) / C::TI;
     const Sched sc = bsym_sched(nchunk, C::CPT, C::TI);
+    const int run = bsym_run(nchunk);
     long long er = 0;
-    for (int t = 0; t < ntile; ++t) er += (nchunk - t * C::CPT + BSYM_RUN - 1) / BSYM_RUN;
+    for (int t = 0; t < ntile; ++t) er += (nchunk - t * C::CPT + run - 1) / run;
     const long long ej = sched_jrow(ntile - 1, sc);
     if ((jcol + ej + (nrun + er) * C::TI) * D > BSYM_MAX_FLOAT2) continue;
     b->sym[e] = 1;
     ens[e] = BEns{(int)runs.size(), ntile, nchunk, 0, jcol};
     for (int t = 0; t < ntile; ++t) {
       runs.push_back(nrun);
-      for (int ca = t * C::CPT; ca < nchunk; ca += BSYM_RUN)
-        units.push_back(BUnit{e, t, ca, std::min(nchunk, ca + BSYM_RUN), nrun++});
+      for (int ca = t * C::CPT; ca < nchunk; ca += run)
+        units.push_back(BUnit{e, t, ca, std::min(nchunk, ca + run), nrun++});
     }
     runs.push_back(nrun);
     jcol += ej;
