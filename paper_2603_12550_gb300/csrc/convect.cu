@@ -15,7 +15,7 @@
 // x 98304 values); in between, every value is read up to four times, once for
 // its own node and once for each neighbour downwind.  k_convect_tile takes a
 // block of up to 64 neighbouring nodes and 128 values per CTA (32 KB), so that
-// most of those reads hit in L1, 16 bytes per lane: 95 -> MEASURED us.
+// most of those reads hit in L1, 16 bytes per lane: 95 -> 72 us.
 // k_convect, one node per CTA with the neighbours' values from L2 (whose
 // bandwidth bound it: four reads of the field in 95 us), is left for values per
 // node that are not a multiple of four and for unaligned arrays: the node is
@@ -100,10 +100,12 @@ __global__ void __launch_bounds__(CV_NT)
 
 constexpr int CT_NODES = 64, CT_NT = 256, CT_COLS = 32;  // nodes, threads, float4 columns per CTA
 
-// Nodes per axis of a CTA's block, powers of two with product <= CT_NODES.
+// A CTA's block of nodes (at most CT_NODES; the last ones of an axis may be
+// cut) and of columns.
 struct CvTile {
-  int lx, ly, lz;  // log2
+  int x, y, z;     // nodes per axis
   int bx, by, bz;  // blocks per axis
+  int lg, cols;    // log2 of the nodes, rounded up; groups of CT_COLS columns
 };
 
 __global__ void __launch_bounds__(CT_NT)
@@ -112,14 +114,14 @@ __global__ void __launch_bounds__(CT_NT)
   __shared__ int s_g[CT_NODES], s_nb[3][CT_NODES];  // node, upwind neighbours; -1: none
   __shared__ float s_u[3][CT_NODES];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nodes = 1 << (T.lx + T.ly + T.lz);
+  const int nodes = 1 << T.lg;
   if (tid < nodes) {
     const int b = blockIdx.x;
-    const int ix = ((b % T.bx) << T.lx) + (tid & ((1 << T.lx) - 1));
-    const int iy = (((b / T.bx) % T.by) << T.ly) + ((tid >> T.lx) & ((1 << T.ly) - 1));
-    const int iz = ((b / (T.bx * T.by)) << T.lz) + (tid >> (T.lx + T.ly));
+    const int ix = (b % T.bx) * T.x + tid % T.x;
+    const int iy = ((b / T.bx) % T.by) * T.y + (tid / T.x) % T.y;
+    const int iz = (b / (T.bx * T.by)) * T.z + tid / (T.x * T.y);
     int g = -1;
-    if (ix < nx && iy < ny && iz < nz) {
+    if (tid < T.x * T.y * T.z && ix < nx && iy < ny && iz < nz) {
       g = ix + nx * (iy + ny * iz);
       // the neighbour that the flow comes from along an axis (periodic or clamped)
       auto up = [&](float v, int i, int n, int stride) -> int {
@@ -141,12 +143,12 @@ __global__ void __launch_bounds__(CT_NT)
     s_g[tid] = g;
   }
   __syncthreads();
-  const long m = ((long)blockIdx.y + (long)gridDim.y * blockIdx.z) * CT_COLS + lane;
-  if (m >= M4) return;
+  const long m0 = ((long)blockIdx.y + (long)gridDim.y * blockIdx.z) * T.cols * CT_COLS + lane;
   auto upd = [](float d, float ub, float c, float v) { return d + (ub > 0.f ? ub * (c - v) : ub * (v - c)); };
-  for (int n = warp; n < nodes; n += CT_NT / 32) {
-    const int g = s_g[n];
-    if (g < 0) continue;
+  for (int x = warp; x < nodes * T.cols; x += CT_NT / 32) {
+    const int n = x & (nodes - 1), g = s_g[n];
+    const long m = m0 + (long)(x >> T.lg) * CT_COLS;
+    if (g < 0 || m >= M4) continue;
     const float4 c = q[(size_t)g * M4 + m];
     float4 v[3], d = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -182,8 +184,41 @@ extern "C" int vds_convect(vds_ctx *c, const float *q_in, float *q_out, int nx, 
   if (cudaGetDevice(&prev) != cudaSuccess) return VDS_ECUDA;
   if (prev != c->device && cudaSetDevice(c->device) != cudaSuccess) return VDS_ECUDA;
   const bool wide = M % 4 == 0 && ((size_t)q_in | (size_t)q_out) % 16 == 0;
+  CvTile T = {1, 1, 1, 1, 1, 1, 0, 1};
   const int per = wide ? 4 * CT_COLS : CV_NT * CV_PER;
-  const long chunks = (M + per - 1) / per;
+  long chunks = (M + per - 1) / per;
+  if (wide) {
+    // block of nodes: double the shortest axis that has nodes left; small
+    // fields take smaller blocks (a node per warp at least) to use every SM
+    int most = CT_NODES, len[3] = {1, 1, 1};
+    const int n[3] = {nx, ny, nz};
+    while (most > CT_NT / 32 && G / most * chunks < 2 * c->num_sms) most /= 2;
+    for (;;) {
+      int best = -1;
+      for (int a = 0; a < 3; ++a)
+        if (len[a] < n[a] && (best < 0 || len[a] < len[best])) best = a;
+      if (best < 0 || 2 * len[0] * len[1] * len[2] > most) break;
+      len[best] *= 2;
+    }
+    // blocks of an axis equally long: 9 nodes are 5 and 4, not 8 and 1 (9 x 9
+    // nodes x 98304 values 16.7 -> 12.7 us)
+    int blk[3];
+    for (int a = 0; a < 3; ++a) {
+      blk[a] = (n[a] + len[a] - 1) / len[a];
+      len[a] = (n[a] + blk[a] - 1) / blk[a];
+    }
+    T = CvTile{len[0], len[1], len[2], blk[0], blk[1], blk[2], 0, 1};
+    while (1 << T.lg < T.x * T.y * T.z) ++T.lg;
+    // a block of few nodes takes more columns, so that a CTA still has CT_NODES
+    // rows of 32 columns to move, while eight CTAs per SM remain (values per
+    // node 8 Mi; k_convect / 32 columns always / this: one node 17 / 107 / 10.5
+    // us, 12 in a row 173 / 308 / 136, 5 x 5 360 / 710 / 315)
+    const long blocks = (long)blk[0] * blk[1] * blk[2];
+    while ((T.cols << T.lg) < CT_NODES && blocks * chunks >= 16L * c->num_sms) {
+      T.cols *= 2;
+      chunks = (chunks + 1) / 2;
+    }
+  }
   const unsigned gy = (unsigned)(chunks < 65535 ? chunks : 65535);
   const long gz = (chunks + gy - 1) / gy;
   int st = VDS_OK;
@@ -192,23 +227,6 @@ extern "C" int vds_convect(vds_ctx *c, const float *q_in, float *q_out, int nx, 
   } else {
     const float cx = (float)(dt / dx[0]), cy = (float)(dt / dx[1]), cz = (float)(dt / dx[2]);
     if (wide) {
-      // block of nodes: double the shortest axis that has nodes left; small
-      // fields take smaller blocks (a node per warp at least) to use every SM
-      int most = CT_NODES;
-      while (most > CT_NT / 32 && G / most * chunks < 2 * c->num_sms) most /= 2;
-      CvTile T = {0, 0, 0, 0, 0, 0};
-      for (;;) {
-        int *const l[3] = {&T.lx, &T.ly, &T.lz};
-        const int n[3] = {nx, ny, nz};
-        int best = -1;
-        for (int a = 0; a < 3; ++a)
-          if ((1 << *l[a]) < n[a] && (best < 0 || *l[a] < *l[best])) best = a;
-        if (best < 0 || (2 << (T.lx + T.ly + T.lz)) > most) break;
-        ++*l[best];
-      }
-      T.bx = (nx + (1 << T.lx) - 1) >> T.lx;
-      T.by = (ny + (1 << T.ly) - 1) >> T.ly;
-      T.bz = (nz + (1 << T.lz) - 1) >> T.lz;
       k_convect_tile<<<dim3((unsigned)T.bx * T.by * T.bz, gy, (unsigned)gz), CT_NT, 0, c->stream>>>(
           (const float4 *)q_in, (float4 *)q_out, nx, ny, nz, M / 4, T, u, cx, cy, cz, bc);
     } else {
