@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(DT_NT, 1)
 #pragma unroll
       for (int h = 0; h < DT_CW / 8; ++h) {
         uint32_t(&w)[8] = v[h & 1];
-        tc_wait_ld();
+        tc_wait_ld(w);
         if (h + 1 < DT_CW / 8) tc_ld8_start(ta + (uint32_t)(h * 8 + 8), v[(h + 1) & 1]);
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
