@@ -78,19 +78,21 @@ constexpr size_t DT_SMEM = (size_t)DT_NS * DT_AB + 2 * (size_t)DT_BB;
 constexpr size_t DT_ROW_BYTES = (size_t)1 << 30;  // row sums of one launch
 
 // Tiles (column tile c, row tile r <= 2 c + 1), c in [c0, c1), column tile
-// major: first one of column tile c.  G CTAs take equal contiguous ranges.
+// major: first one of column tile c.  G CTAs take equal contiguous ranges.  The
+// tiles of a launch are at most DT_ROW_BYTES / 512 and those of one column tile,
+// times G below 2^32: 64-bit divisions took a microsecond of a small cloud's pass.
 struct DtSched {
   int c0, c1, G, maxseg;
-  long long items;
+  unsigned items;
 };
-__host__ __device__ __forceinline__ long long dt_start(int c, const DtSched &s) {
-  return (long long)c * (c + 1) - (long long)s.c0 * (s.c0 + 1);
+__host__ __device__ __forceinline__ unsigned dt_start(int c, const DtSched &s) {
+  return (unsigned)((long long)c * (c + 1) - (long long)s.c0 * (s.c0 + 1));
 }
 // First row sum of column tile c (its rows are the 256 c before it).
 __host__ __device__ __forceinline__ size_t dt_row(int c, const DtSched &s) {
   return (size_t)(DT_N / 2) * ((size_t)c * (c - 1) - (size_t)s.c0 * (s.c0 - 1));
 }
-__host__ __device__ __forceinline__ int dt_cta_of(long long x, const DtSched &s) {
+__host__ __device__ __forceinline__ int dt_cta_of(unsigned x, const DtSched &s) {
   return (int)(((x + 1) * s.G + s.items - 1) / s.items - 1);
 }
 
@@ -139,20 +141,22 @@ __global__ void __launch_bounds__(256)
                 int *err) {
   __shared__ float2 ps[8][32];
   const int p = threadIdx.x & 31, u = threadIdx.x >> 5, i = blockIdx.x * 32 + p;
-  vds_pair::Sum2 s;
   const int ci = i / DT_N;
-  if (i < N)
+  vds_pair::Sum2 s;
+  if (i < N) {
     for (int c = max(ci + 1, sc.c0) + u; c < sc.c1; c += 8) s.add(make_float2(rowp[dt_row(c, sc) + i], 0.f));
+    if (ci >= sc.c0 && ci < sc.c1) {  // four quarters of each CTA's part of the column tile: 72 at N = 4097
+      const int f = dt_cta_of(dt_start(ci, sc), sc), l = dt_cta_of(dt_start(ci + 1, sc) - 1, sc);
+      const float2 *col = colp + (size_t)(ci - sc.c0) * sc.maxseg * 4 * DT_N + (i - ci * DT_N);
+#pragma unroll 4
+      for (int g = u; g < 4 * (l - f + 1); g += 8) s.add(col[(size_t)g * DT_N]);
+    }
+  }
   ps[u][p] = make_float2(s.s, s.c);
   __syncthreads();
   if (u || i >= N) return;
   vds_pair::Sum2 t;
   if (!first) t.add(run[i]);
-  if (ci >= sc.c0 && ci < sc.c1) {
-    const int f = dt_cta_of(dt_start(ci, sc), sc), l = dt_cta_of(dt_start(ci + 1, sc) - 1, sc);
-    for (int g = 0; g < 4 * (l - f + 1); ++g)
-      t.add(colp[((size_t)(ci - sc.c0) * sc.maxseg * 4 + g) * DT_N + (i - ci * DT_N)]);
-  }
   for (int v = 0; v < 8; ++v) t.add(ps[v][p]);
   if (!last) {
     run[i] = make_float2(t.s, t.c);
@@ -230,7 +234,7 @@ __global__ void __launch_bounds__(DT_NT, 1)
   __shared__ int s_abort;
   __shared__ float s_row[DT_RS][DT_HC][DT_M];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long g0 = (long long)blockIdx.x * sc.items / sc.G, g1 = (long long)(blockIdx.x + 1) * sc.items / sc.G;
+  const unsigned g0 = blockIdx.x * sc.items / sc.G, g1 = (blockIdx.x + 1) * sc.items / sc.G;
   const int nt = (int)(g1 - g0);
   // the range's first column and row tile
   int cb = sc.c0, re = sc.c1;
@@ -487,7 +491,7 @@ int dens_tc_impl(vds_ctx *c, int N, float *rho_out) {
     sc.c1 = c0 + 1;
     while (sc.c1 < ntc && dt_row(sc.c1 + 1, sc) * sizeof(float) <= DT_ROW_BYTES) ++sc.c1;
     sc.items = dt_start(sc.c1, sc);
-    sc.G = (int)(sc.items < c->num_sms ? sc.items : c->num_sms);
+    sc.G = sc.items < (unsigned)c->num_sms ? (int)sc.items : c->num_sms;
     sc.maxseg = 1;
     for (int t = sc.c0; t < sc.c1; ++t) {
       const int n = dt_cta_of(dt_start(t + 1, sc) - 1, sc) - dt_cta_of(dt_start(t, sc), sc) + 1;
