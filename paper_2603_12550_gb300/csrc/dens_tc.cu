@@ -75,7 +75,8 @@ constexpr int DT_BB = DT_N * DT_RB;        // 32 KB
 constexpr int DT_RS = 4;                   // row-sum buffers
 constexpr int DT_FOLD = 64;                // row tiles between two folds of the column sums
 constexpr size_t DT_SMEM = (size_t)DT_NS * DT_AB + 2 * (size_t)DT_BB;
-constexpr size_t DT_ROW_BYTES = (size_t)1 << 30;  // row sums of one launch
+constexpr size_t DT_ROW_BYTES = (size_t)1 << 30;  // row sums of one launch ...
+constexpr size_t DT_ROW_LEAST = (size_t)1 << 23;  // ... or down to this many where memory is short
 
 // Tiles (column tile c, row tile r <= 2 c + 1), c in [c0, c1), column tile
 // major: first one of column tile c.  G CTAs take equal contiguous ranges.  The
@@ -484,12 +485,13 @@ int dens_tc_impl(vds_ctx *c, int N, float *rho_out) {
   const int Npad = (N + DT_N - 1) / DT_N * DT_N;
   const int ntc = Npad / DT_N;
   const size_t img = (size_t)Npad * DT_RB;
-  // a launch's column tiles from c0 on: as many as DT_ROW_BYTES hold
+  // a launch's column tiles from c0 on: as many as `limit` bytes of row sums hold
+  size_t limit = DT_ROW_BYTES;
   auto sched = [&](int c0) {
     DtSched sc;
     sc.c0 = c0;
     sc.c1 = c0 + 1;
-    while (sc.c1 < ntc && dt_row(sc.c1 + 1, sc) * sizeof(float) <= DT_ROW_BYTES) ++sc.c1;
+    while (sc.c1 < ntc && dt_row(sc.c1 + 1, sc) * sizeof(float) <= limit) ++sc.c1;
     sc.items = dt_start(sc.c1, sc);
     sc.G = sc.items < (unsigned)c->num_sms ? (int)sc.items : c->num_sms;
     sc.maxseg = 1;
@@ -499,16 +501,23 @@ int dens_tc_impl(vds_ctx *c, int N, float *rho_out) {
     }
     return sc;
   };
-  size_t rowb = 0, colb = 0;
-  for (int c0 = 0; c0 < ntc;) {
-    const DtSched sc = sched(c0);
-    const size_t r = dt_row(sc.c1, sc) * sizeof(float);
-    const size_t l = (size_t)(sc.c1 - sc.c0) * sc.maxseg * 4 * DT_N * sizeof(float2);
-    if (r > rowb) rowb = r;
-    if (l > colb) colb = l;
-    c0 = sc.c1;
+  size_t rowb, colb;
+  for (;;) {
+    rowb = colb = 0;
+    for (int c0 = 0; c0 < ntc;) {
+      const DtSched sc = sched(c0);
+      const size_t r = dt_row(sc.c1, sc) * sizeof(float);
+      const size_t l = (size_t)(sc.c1 - sc.c0) * sc.maxseg * 4 * DT_N * sizeof(float2);
+      if (r > rowb) rowb = r;
+      if (l > colb) colb = l;
+      c0 = sc.c1;
+    }
+    const int st = vds_ensure(c, c->dtbuf, 2 * img + colb + (size_t)N * sizeof(float2) + rowb);
+    if (st == VDS_OK) break;
+    if (st != VDS_ENOMEM || limit <= DT_ROW_LEAST) return st;
+    (void)cudaGetLastError();
+    limit = (rowb < limit ? rowb : limit) / 4;  // more launches of fewer column tiles
   }
-  VDS_TRY(vds_ensure(c, c->dtbuf, 2 * img + colb + (size_t)N * sizeof(float2) + rowb));
   uint8_t *aimg = (uint8_t *)c->dtbuf.ptr, *bimg = aimg + img;
   float2 *colp = (float2 *)(bimg + img), *run = (float2 *)((uint8_t *)colp + colb);
   float *rowp = (float *)(run + N);

@@ -52,8 +52,14 @@ int vds_ensure(vds_ctx *c, DevBuf &b, size_t bytes) {
     b.ptr = nullptr;
     b.cap = 0;
   }
-  const size_t want = bytes + bytes / 4 + 256;
-  VDS_CUDA_TRY(cudaMalloc(&b.ptr, want));
+  size_t want = bytes + bytes / 4 + 256;
+  cudaError_t e = cudaMalloc(&b.ptr, want);
+  if (e == cudaErrorMemoryAllocation) {  // without the room to grow
+    (void)cudaGetLastError();
+    want = bytes;
+    e = cudaMalloc(&b.ptr, want);
+  }
+  VDS_CUDA_TRY(e);
   b.cap = want;
   return VDS_OK;
 }
