@@ -16,7 +16,16 @@
  *    call synchronises the context stream before returning them.  Every other
  *    call is asynchronous on the context stream.
  *  - The library owns the context (its stream binding and device workspace)
- *    and pod_basis objects.
+ *    and pod_basis objects.  The workspace grows on demand and is held until
+ *    vds_destroy.  Its large parts grow with N^2: partial sums of the passes
+ *    over unordered pairs (about N^2 / 4608 x 8 D bytes for N >= 49152, three times
+ *    that below, at most 4 GiB: 67 MB at N = 65536, D = 9), of the tensor-core
+ *    density (N^2 / 128 bytes, at most 1 GiB) and the keys of the median
+ *    bandwidth (at most 1 GiB: 63 MB at N = 65536), up to a quarter more each
+ *    as room to grow.  The first and the last are taken only within a quarter
+ *    of the memory that is free on the device at that time, the second in
+ *    smaller pieces where it cannot be had; the calls work without them, more
+ *    slowly.
  *  - Return value: VDS_OK or a negative status; on error the outputs are
  *    unspecified and no memory is leaked.  Device-side failures (a FENE bond
  *    leaving |q|^2 < b, a NaN, a wait that gave up) are reported by the next

@@ -35,7 +35,11 @@ typedef struct vds_batch vds_batch;
 /* Set up a batch of E ensembles: sizes (host, E ints, each >= 1), h (host,
  * E doubles > 0), kappa (host, E x s x s doubles, row-major per ensemble),
  * shared parameters p (p->h and p->kappa are ignored).  D = p->nb * p->s.
- * The batch owns its device workspace. */
+ * The batch owns its device workspace: about 40 bytes per coordinate, and for
+ * the ensembles over unordered pairs partial sums of 4 to 33 MB per 16384
+ * particles of one ensemble (quadratic in its size), at most 4 GiB and a quarter
+ * of the device's free memory at creation, beyond which ensembles stay with the
+ * ordered items. */
 VDS_API int vds_batch_create(vds_ctx *ctx, int E, const int *sizes, int D, const vds_params *p,
                              const double *h, const double *kappa, vds_batch **out);
 VDS_API void vds_batch_free(vds_batch *b);

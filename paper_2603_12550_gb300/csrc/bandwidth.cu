@@ -139,6 +139,7 @@ __global__ void k_sel_digit(SelState *st, unsigned long long *ghist, int pass, l
 // ------------------------------------------------- bracketed selection
 
 constexpr unsigned long long SMALL_PAIRS = 1ull << 22;
+constexpr unsigned long long MOST_KEYS = 1ull << 28;  // 1 GiB of workspace: clouds of about a million particles
 constexpr int SEL_NT = 512, SEL_BINS = 2048, SEL_BITS = 11;
 
 // Selection of up to two order statistics among keys in [lo, hi], by digits of
@@ -562,14 +563,17 @@ int select_impl(vds_ctx *c, const float *q, int N, bool &done) {
   done = false;
   const unsigned long long M = num_pairs(N), rank = (M - 1ull) / 2ull;
   const bool small = M <= SMALL_PAIRS;
+  // sample: from (7.5 M)^(2/3) on (N above 350000) it would hold more keys than
+  // the bracket it gives
   unsigned long long n = M / 1024;
+  if (n > (1ull << 20)) n = (unsigned long long)fmin((double)n, cbrt(7.5 * (double)M) * cbrt(7.5 * (double)M));
   if (n < (1ull << 20)) n = 1ull << 20;
   const double half = 2.5 * sqrt((double)n);
   // room for the sample, then for half as many keys again as the bracket holds on average
   const unsigned long long want = small ? M : (unsigned long long)(1.5 * 2.0 * half / (double)n * (double)M);
   const unsigned long long cap = small ? M : (want > n ? want : n);
   VDS_TRY(vds_ensure(c, c->red, sizeof(Sel) + 2 * SEL_BINS * sizeof(unsigned)));
-  int st = vds_ensure(c, c->part, cap * sizeof(unsigned));
+  int st = cap <= MOST_KEYS ? vds_ensure_spare(c, c->part, cap * sizeof(unsigned)) : VDS_ENOMEM;
   if (st == VDS_OK && !small) st = vds_ensure(c, c->rec, (size_t)N * Scr<D>::DP * sizeof(float));
   if (st == VDS_ENOMEM) {
     (void)cudaGetLastError();

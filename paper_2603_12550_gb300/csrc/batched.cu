@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(NT)
 // tiles of 1024 is three tile pairs' work where the ordered form has four.
 constexpr int BSYM_MIN_N = 2048;
 constexpr int BSYM_TJS = 32, BSYM_NT = 128;
-constexpr long long BSYM_MAX_FLOAT2 = (long long)1 << 29;  // workspace: 4 GiB
+constexpr long long BSYM_MAX_FLOAT2 = (long long)1 << 29;  // workspace: 4 GiB, and a quarter of the free memory
 // j-chunks per unit: a sixteenth of the ensemble, 8 to 32.  The longest unit sets
 // the time of a batch that does not fill the GPU, and long units its last round;
 // shorter ones cost more tile loads and sums.  They follow the ensemble's size
@@ -932,6 +932,9 @@ int b_setup_sym(vds_ctx *c, vds_batch *b) {
   long long jcol = 0;
   int nrun = 0;
   b->sym.assign(b->E, 0);
+  size_t spare = 0;
+  VDS_TRY(vds_spare_bytes(0, &spare));
+  const long long most = std::min(BSYM_MAX_FLOAT2, (long long)(spare / sizeof(float2)));
   for (int e = 0; e < b->E; ++e) {
     const int N = b->sizes[e];
     if (N < BSYM_MIN_N) continue;
@@ -941,7 +944,7 @@ int b_setup_sym(vds_ctx *c, vds_batch *b) {
     long long er = 0;
     for (int t = 0; t < ntile; ++t) er += (nchunk - t * C::CPT + run - 1) / run;
     const long long ej = sched_jrow(ntile - 1, sc);
-    if ((jcol + ej + (nrun + er) * C::TI) * D > BSYM_MAX_FLOAT2) continue;
+    if ((jcol + ej + (nrun + er) * C::TI) * D > most) continue;
     b->sym[e] = 1;
     ens[e] = BEns{(int)runs.size(), ntile, nchunk, 0, jcol};
     for (int t = 0; t < ntile; ++t) {

@@ -499,8 +499,8 @@ struct SymCfg {
   static constexpr int NT_LARGE = MINB128 * 128;  // one CTA per SM
 };
 
-// The j sums of a symmetric pass may take this much workspace; larger clouds
-// (and a workspace that cannot be had) take the ordered form.
+// The j sums of a symmetric pass may take this much workspace, and a quarter of
+// the free memory; beyond either the pass takes the ordered form.
 constexpr size_t SYM_MAX_PARTJ = (size_t)4 << 30;
 // Smaller clouds take k_small.  Explicit step, k_small / symmetric passes:
 // N = 4096, D = 2 25 / 29 us, D = 9 49 / 63, D = 16 72 / 75; N = 6144, D = 3
@@ -553,8 +553,8 @@ int launch_sym(vds_ctx *c, int N, Sched &sc, const ImpState *imp, bool &done) {
   sc.maxseg = sched_maxseg(sc);
   const size_t jbytes = (size_t)sched_jrow(sc.n_itiles - 1, sc) * ACC * sizeof(float2);
   if (jbytes > SYM_MAX_PARTJ) return VDS_OK;
-  int st = vds_ensure(c, c->part, (size_t)sc.n_itiles * sc.maxseg * TI * ACC * sizeof(float2));
-  if (st == VDS_OK && jbytes) st = vds_ensure(c, c->partj, jbytes);
+  int st = jbytes ? vds_ensure_spare(c, c->partj, jbytes) : VDS_OK;
+  if (st == VDS_OK) st = vds_ensure(c, c->part, (size_t)sc.n_itiles * sc.maxseg * TI * ACC * sizeof(float2));
   if (st == VDS_ENOMEM) {
     (void)cudaGetLastError();
     return VDS_OK;

@@ -64,6 +64,25 @@ int vds_ensure(vds_ctx *c, DevBuf &b, size_t bytes) {
   return VDS_OK;
 }
 
+int vds_spare_bytes(size_t held, size_t *bytes) {
+  size_t free_b = 0, total = 0;
+  VDS_CUDA_TRY(cudaMemGetInfo(&free_b, &total));
+  *bytes = (free_b + held) / 4;
+  return VDS_OK;
+}
+
+int vds_ensure_spare(vds_ctx *c, DevBuf &b, size_t bytes) {
+  if (bytes <= b.cap) return VDS_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return VDS_ENOMEM;
+  }
+  size_t most = 0;
+  VDS_TRY(vds_spare_bytes(b.cap, &most));
+  return bytes + bytes / 4 + 256 <= most ? vds_ensure(c, b, bytes) : VDS_ENOMEM;
+}
+
 static int timing_harvest(vds_ctx *c) {
   TimingPool *t = c->timing;
   if (!t) return VDS_OK;

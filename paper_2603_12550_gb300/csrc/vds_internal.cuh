@@ -229,6 +229,12 @@ struct vds_ctx {
 };
 
 int vds_ensure(vds_ctx *c, DevBuf &b, size_t bytes);
+// The same for a large buffer that its user can do without: VDS_ENOMEM, and
+// nothing changed, where it would take more than a quarter of the device's free
+// memory (vds_spare_bytes, what the buffer holds counted as free), so that the
+// program around the library keeps the rest, and while the stream is captured.
+int vds_ensure_spare(vds_ctx *c, DevBuf &b, size_t bytes);
+int vds_spare_bytes(size_t held, size_t *bytes);
 // Bracket a pair-pass launch of kind `pk` with timing events (no-op unless
 // instrumentation is on).
 int vds_time_begin(vds_ctx *c, int pk);
