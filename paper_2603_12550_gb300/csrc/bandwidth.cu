@@ -11,9 +11,10 @@
 //      below lo and collects those inside, about 160 sqrt(M) of them;
 //   3. an exact radix select among the collected keys.
 // Where the bracket misses the median (by the counts of step 2; once in 10^6
-// clouds, or with many equal distances), or a particle lies so far out that
-// the screen of step 2 has no resolution, a radix select by three histogram
-// passes over all pairs (k_hist) takes over.  Clouds of up to SMALL_PAIRS
+// clouds), or the sample shows many equal distances, or a particle lies so far
+// out that the screen of step 2 has no resolution, or the keys take more room
+// than there is (from about a million particles on), a radix select by three
+// histogram passes over all pairs (k_hist) takes over.  Clouds of up to SMALL_PAIRS
 // pairs write all keys and select among them.
 //
 // The FP32 and integer issue bounds step 2.  It screens the pairs by
@@ -146,7 +147,7 @@ constexpr int SEL_NT = 512, SEL_BINS = 2048, SEL_BITS = 11;
 // key - lo: what has been found so far (prefix) and the rank left inside it.
 struct Sel {
   unsigned lo, hi;              // the bracket
-  unsigned prefix[2];
+  unsigned prefix[2], count[2];  // count: keys with the prefix
   unsigned long long rank[2];
   unsigned long long below;     // pairs with a key below lo
   unsigned long long in;        // pairs with a key in the bracket
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(SEL_NT)
       for (int k = 0; k < PT; ++k) {
         if (rank >= base && rank < base + c[k]) {
           s->rank[t] = rank - base;
+          s->count[t] = (unsigned)c[k];
           s->prefix[t] = level ? (s->prefix[t] << (up - sh)) | (unsigned)(tid * PT + k) : (unsigned)(tid * PT + k);
         }
         base += c[k];
@@ -345,23 +347,30 @@ __global__ void k_screen_rec(const float *__restrict__ q, int N, Sel *s, float *
   if ((threadIdx.x & 31) == 0) atomicMax(&s->ymax2, m);
 }
 
-// The bracket from the two prefixes found in the sample (two levels of a
-// 32-bit span: the top 22 bits), the state of the pass that uses it, and the
-// screen's.  With u = 2^-24 and Y^2 >= |y|^2 for every particle, the screen
-// value differs from the key's float (both of the pair's true squared
+// The bracket from the two prefixes that `levels` levels of a 32-bit span found in
+// the sample of n keys (order statistics r0 and r1), the state of the pass that
+// uses it, and the screen's.  With u = 2^-24 and Y^2 >= |y|^2 for every particle,
+// the screen value differs from the key's float (both of the pair's true squared
 // distance) by at most
 //   2D u Y^2 (the norms) + 5 u Y^2 (|y_i|^2 - slo) + 6 u Y^2 (their sum) +
 //   8D u Y^2 (D fused steps of partial sums up to 8 Y^2) + 8 u Y^2 (rounding
 //   y) + 4 (D + 2) u Y^2 (the key)  =  (14D + 27) u Y^2.
-__global__ void k_sel_bracket(Sel *s, int D) {
-  const int sh = sel_shift(0xffffffffu, 1);
+// A miss at once where the sample says that the bracket holds more keys than
+// there is room for (equal distances), or that the widened one holds over 2 % of
+// the pairs, as the queue of the pass then takes longer than the histograms save.
+__global__ void k_sel_bracket(Sel *s, int D, int levels, unsigned long long r0, unsigned long long r1,
+                              unsigned long long n, unsigned long long M, unsigned long long cap) {
+  const int sh = sel_shift(0xffffffffu, levels - 1);
   s->lo = s->prefix[0] << sh;
   s->hi = (s->prefix[1] << sh) | ((1u << sh) - 1u);
   s->prefix[0] = 0u;
   const double lo = __uint_as_float(s->lo), hi = __uint_as_float(s->hi), y2 = __uint_as_float(s->ymax2);
   const double eps = (14.0 * D + 40.0) * 5.9604644775390625e-8 * y2 * 1.0001;
-  // worth it while it widens the bracket by less than a quarter
-  if (!(y2 < 1e30 && hi < 1e30 && eps <= 0.125 * (hi - lo))) s->miss = 1u;
+  // part of the sample, and so of the pairs, inside
+  const double in = (double)((r1 - s->rank[1] + s->count[1]) - (r0 - s->rank[0])) / (double)n;
+  const double width = hi > lo ? hi - lo : 0.0;
+  if (!(y2 < 1e30 && hi < 1e30 && in * (double)M <= 0.99 * (double)cap && in * (width + 2.0 * eps) <= 0.02 * width))
+    s->miss = 1u;
   s->slo = __double2float_rd(lo - eps);
   s->sspan = __double2float_ru((hi + eps) - (double)s->slo);
 }
@@ -597,14 +606,17 @@ int select_impl(vds_ctx *c, const float *q, int N, bool &done) {
     for (int l = 0; l < 3; ++l) level((long)M, M, l, 1);
     c->launches += 2;
   } else {
-    k_sel_start<<<1, 512, 0, c->stream>>>(s, gh, (unsigned long long)(0.5 * (double)n - half),
-                                          (unsigned long long)(0.5 * (double)n + half));
+    const unsigned long long r0 = (unsigned long long)(0.5 * (double)n - half),
+                             r1 = (unsigned long long)(0.5 * (double)n + half);
+    // the top 22 bits of the keys resolve the bracket of a small sample
+    const int levels = n > (1ull << 23) ? 3 : 2;
+    k_sel_start<<<1, 512, 0, c->stream>>>(s, gh, r0, r1);
     k_sample<D><<<8 * c->num_sms, 256, 0, c->stream>>>(q, N, (long)n, keys);
-    for (int l = 0; l < 2; ++l) level((long)n, n, l, 2);
+    for (int l = 0; l < levels; ++l) level((long)n, n, l, 2);
     k_centre<D><<<1, 512, 0, c->stream>>>(q, N, s);
     float *rec = (float *)c->rec.ptr;
     k_screen_rec<D><<<(N + 255) / 256, 256, 0, c->stream>>>(q, N, s, rec);
-    k_sel_bracket<<<1, 1, 0, c->stream>>>(s, D);
+    k_sel_bracket<<<1, 1, 0, c->stream>>>(s, D, levels, r0, r1, n, M, cap);
     using C = BrCfg<D>;
     Sched sc;
     sc.TI = C::TI;
@@ -621,7 +633,7 @@ int select_impl(vds_ctx *c, const float *q, int N, bool &done) {
     VDS_TRY(vds_time_end(c, PK_BANDWIDTH));
     k_sel_collected<<<1, 1, 0, c->stream>>>(s, rank, cap);
     for (int l = 0; l < 3; ++l) level(-1, (unsigned long long)(2.0 * half / (double)n * (double)M), l, 1);
-    c->launches += 7;
+    c->launches += 5 + levels;
   }
   k_sel_done<<<1, 1, 0, c->stream>>>(s, N, c->scal);
   ++c->launches;
