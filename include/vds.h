@@ -232,8 +232,11 @@ VDS_API int vds_energy_grad_noalloc(const float *q, int N, int D, const vds_para
 
 /* Instrumentation (no counterpart in the paper; used to report a kernel's
  * achieved rate).  vds_timing(ctx, 1) clears the counters and starts
- * recording the device duration of every pair-pass launch and POD phase on
- * the context stream (CUDA events around it); vds_timing(ctx, 0) stops.  The
+ * recording the device duration of every pair-pass launch (a small cloud's
+ * pass and its epilogue are one launch) and POD phase on the context stream
+ * (CUDA events around it); vds_timing(ctx, 0) stops.  Explicit steps are then
+ * launched one by one, and implicit steps read the minimiser's state back
+ * after every pass, so that only evaluations are counted.  The
  * library's total kernel-launch count is cleared by either call.
  * vds_timing_read synchronises and returns, per kind, the summed milliseconds
  * ms[VDS_TIMING_KINDS] and event-pair counts launches[VDS_TIMING_KINDS] (host

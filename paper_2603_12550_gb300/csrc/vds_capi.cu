@@ -430,9 +430,12 @@ static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
 // seven evaluations, the 2D dumbbell at N = 512 took 300-400 us a step, two
 // thirds of it host round trips.  The host enqueues rounds of (trial point,
 // density, gradient) without looking; those that are not due return at once
-// (about 2 us).  Most steps need two gradients: two rounds per step are
-// enqueued, a step that needs more goes on in the rounds meant for the next,
-// and what is missing at the end is enqueued then.
+// (about 2 us).  Most steps need two gradients: two rounds per step are enqueued
+// for N > 16384, three below (four in a call's first step and from the 65th on),
+// a step that needs more goes on in the rounds meant for the next, and what is
+// missing at the end is enqueued then.  With phase timing on the state is read
+// back after every pass and only what is due is launched, so that the counts are
+// those of the evaluations; the results are the same bits.
 static int step_implicit(vds_ctx *c, float *q, const KParams &kp, const vds_params *p, int nsteps,
                          int *iters_out) {
   const size_t nd = (size_t)kp.N * kp.D;
@@ -461,17 +464,37 @@ static int step_implicit(vds_ctx *c, float *q, const KParams &kp, const vds_para
     VDS_TRY(imp_trial(c, kp, imp, qs, dir));  // for a step that goes on
     return imp_end(c, kp, imp, qs, dir, q, iters);
   };
+  auto finish = [&](int st) -> int {
+    if (iters_out && s.step > 0)
+      VDS_CUDA_TRY(cudaMemcpy(iters_out, iters, (size_t)s.step * sizeof(int), cudaMemcpyDeviceToHost));
+    return st != VDS_OK ? st : s.status;
+  };
+  auto read_state = [&]() -> int {
+    VDS_CUDA_TRY(cudaMemcpyAsync(&s, imp.st, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
+    return vds_sync_status(c);
+  };
+  if (c->timing && c->timing->on) {
+    int st = VDS_OK;
+    while (st == VDS_OK && s.phase != IMP_STOP && s.step < nsteps) {
+      if (s.phase == IMP_GRAD) {
+        VDS_TRY(pass_grad(c, kp, GM_IMPLICIT_DIR, dir, qs, nullptr, nullptr, nullptr, nullptr, &imp));
+      } else if (s.phase == IMP_FINAL) {
+        VDS_TRY(imp_end(c, kp, imp, qs, dir, q, iters));
+      } else {
+        if (s.phase == IMP_READY) VDS_TRY(imp_begin(c, kp, imp, q, qs));
+        else VDS_TRY(imp_trial(c, kp, imp, qs, dir));
+        VDS_TRY(pass_density(c, kp, nullptr, true, qs, nullptr, nullptr, nullptr, &imp));
+      }
+      st = read_state();
+    }
+    return finish(st);
+  }
   for (bool first = true;; first = false) {
     // at most this many steps ahead of the host
     const int ahead = nsteps - s.step < 64 ? nsteps - s.step : 64;
     for (int k = 0; k < ahead; ++k) VDS_TRY(one_step(kp.N > 16384 ? 2 : first && k > 0 ? 3 : 4));
-    VDS_CUDA_TRY(cudaMemcpyAsync(&s, imp.st, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
-    const int st = vds_sync_status(c);
-    if (st != VDS_OK || s.phase == IMP_STOP || s.step >= nsteps) {
-      if (iters_out && s.step > 0)
-        VDS_CUDA_TRY(cudaMemcpy(iters_out, iters, (size_t)s.step * sizeof(int), cudaMemcpyDeviceToHost));
-      return st != VDS_OK ? st : s.status;
-    }
+    const int st = read_state();
+    if (st != VDS_OK || s.phase == IMP_STOP || s.step >= nsteps) return finish(st);
   }
 }
 
