@@ -353,9 +353,10 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int t = 0; t < BT; ++t) {
           const float2 w = Ws[mm][t];
-          const float p = x * w.x, e = fmaf(x, w.x, -p);
-          const float s = hi[t] + p, b = s - hi[t];
-          lo[t] += ((hi[t] - (s - b)) + (p - b)) + fmaf(x, w.y, e);
+          // a contracted product (fma(x, w.x, hi)) would add its rounding twice
+          const float p = __fmul_rn(x, w.x), e = fmaf(x, w.x, -p);
+          const float s = __fadd_rn(hi[t], p), b = __fsub_rn(s, hi[t]);
+          lo[t] += __fadd_rn(__fsub_rn(hi[t], __fsub_rn(s, b)), __fsub_rn(p, b)) + fmaf(x, w.y, e);
           hi[t] = s;
         }
       }
