@@ -186,21 +186,6 @@ __device__ __forceinline__ bool dt_wait(uint64_t *bar, uint32_t parity, volatile
   }
 }
 
-// Two FP32 values per register pair.
-__device__ __forceinline__ unsigned long long f2_pack(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(unsigned long long v, float &a, float &b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // Sums over the warp's lanes of 32 values per lane: lane l returns the sum of value l.
 __device__ __forceinline__ float lane_sums(float (&x)[32], int lane) {
 #pragma unroll

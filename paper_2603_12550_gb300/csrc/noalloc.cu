@@ -159,7 +159,7 @@ int na_energy_grad(const DevState &s, const float *q, const KParams &kp, double 
   const int Npad = (N + TJ - 1) / TJ * TJ;
   // error flag and tickets must start at zero
   VDS_CUDA_TRY(cudaMemsetAsync(base, 0, kScalOff, st));
-  k_prep<D><<<(Npad + 255) / 256, 256, 0, st>>>(N, Npad, kp.c, q, nullptr, nullptr, 0.f, nullptr, rec);
+  k_prep<D><<<(Npad + 255) / 256, 256, 0, st>>>(N, Npad, kp.c, q, rec);
   VDS_CUDA_TRY(cudaGetLastError());
   PartSrc src;
   src.i = part;

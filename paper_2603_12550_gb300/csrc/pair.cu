@@ -53,77 +53,77 @@ __global__ void __launch_bounds__(256)
     default: return VDS_EARG;                            \
   }
 
-int vds_prep_2(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_2(vds_ctx *, const KParams &, const float *);
 int vds_density_2(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_2(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_2(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_2(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_2(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_2(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_3(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_3(vds_ctx *, const KParams &, const float *);
 int vds_density_3(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_3(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_3(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_3(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_3(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_3(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_4(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_4(vds_ctx *, const KParams &, const float *);
 int vds_density_4(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_4(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_4(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_4(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_4(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_4(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_6(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_6(vds_ctx *, const KParams &, const float *);
 int vds_density_6(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_6(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_6(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_6(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_6(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_6(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_8(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_8(vds_ctx *, const KParams &, const float *);
 int vds_density_8(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_8(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_8(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_8(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_8(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_8(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_9(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_9(vds_ctx *, const KParams &, const float *);
 int vds_density_9(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_9(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_9(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_9(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_9(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_9(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_10(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_10(vds_ctx *, const KParams &, const float *);
 int vds_density_10(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_10(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_10(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_10(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_10(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_10(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_12(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_12(vds_ctx *, const KParams &, const float *);
 int vds_density_12(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_12(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_12(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_12(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_12(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_12(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_14(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_14(vds_ctx *, const KParams &, const float *);
 int vds_density_14(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_14(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_14(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_14(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_14(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_14(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_15(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_15(vds_ctx *, const KParams &, const float *);
 int vds_density_15(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_15(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_15(vds_ctx *, const KParams &, const float *, double *, double *);
 int vds_impbegin_15(vds_ctx *, const KParams &, const ImpArgs &, const float *, float *);
 int vds_imptrial_15(vds_ctx *, const KParams &, const ImpArgs &, const float *, const float *);
 int vds_query_15(vds_ctx *, const KParams &, const float *, const float *, int, float *);
-int vds_prep_16(vds_ctx *, const KParams &, const float *, const float *, const float *, float, float *);
+int vds_prep_16(vds_ctx *, const KParams &, const float *);
 int vds_density_16(vds_ctx *, const KParams &, float *, bool, const float *, const float *, const float *, const float *, const ImpArgs *);
 int vds_grad_16(vds_ctx *, const KParams &, int, float *, const float *, const float *, const float *, const float *, float *, const ImpArgs *);
 int vds_stress_16(vds_ctx *, const KParams &, const float *, double *, double *);
@@ -180,9 +180,8 @@ KParams make_kparams(const vds_params *p, int N, int D) {
 
 int pass_npad(int N) { return (N + vds_pair::TJ - 1) / vds_pair::TJ * vds_pair::TJ; }
 
-int pass_prep(vds_ctx *c, const KParams &kp, const float *base, const float *delta,
-              const float *dir, float alpha, float *delta_out) {
-#define CALL(DD) vds_prep_##DD(c, kp, base, delta, dir, alpha, delta_out)
+int pass_prep(vds_ctx *c, const KParams &kp, const float *y) {
+#define CALL(DD) vds_prep_##DD(c, kp, y)
   VDS_DISPATCH_D(kp.D, CALL)
 #undef CALL
 }

@@ -88,15 +88,12 @@ struct KParams {
 
 KParams make_kparams(const vds_params *p, int N, int D);
 
-// Records of y = base + delta (delta may be NULL) scaled by c, with w = 0,
-// padded to Npad with padding records.  If delta_out != NULL it receives
-// delta - alpha*dir (and the record is built from base + that).
 // Rows of the record array written by pass_prep for N particles: N rounded
-// up to the pair passes' j-tile, the rows beyond N far away (kernel value 0)
-// with w = 0.
+// up to the pair passes' j-tile.
 int pass_npad(int N);
-int pass_prep(vds_ctx *c, const KParams &kp, const float *base, const float *delta,
-              const float *dir, float alpha, float *delta_out);
+// Records of y scaled by c, with w = 0, in ctx->rec; the rows beyond N far away
+// (kernel value 0).
+int pass_prep(vds_ctx *c, const KParams &kp, const float *y);
 
 // Density pass: rho_I over all J, then the epilogue: w_I = 1/rho_I into the
 // records, optional rho output, and when want_energy, the FP64 energy
@@ -128,9 +125,9 @@ enum GradMode { GM_OUT = 0, GM_EXPLICIT = 1, GM_IMPLICIT_DIR = 2, GM_VEL = 3 };
 // GM_OUT: g = kBT S + grad Psi(y) (+ (zeta/dt)(A^-1 (x) I)(qa - qb) if qa).
 // GM_EXPLICIT: q_io += dt [kappa q - (1/zeta)(A (x) I) g]; rebuild records.
 // GM_VEL: out = kappa y - (1/zeta)(A (x) I) g (the particle velocity).
-// GM_IMPLICIT_DIR: dir = d + (dt/zeta)(A (x) I) g with d = ydelta, and
-//   scal[SC_DEC] = (1/N) sum <G, dir>, G = (zeta/dt)(A^-1 (x) I) d + g,
-//   scal[SC_DMAX] = max|dir|, scal[SC_YMAX] = max|y|.
+// GM_IMPLICIT_DIR: dir = d + (dt/zeta)(A (x) I) g with d the minimiser's accepted
+//   displacement; its state takes (1/N) sum <G, dir>, G = (zeta/dt)(A^-1 (x) I) d
+//   + g, max|dir| and max|y|.
 int pass_grad(vds_ctx *c, const KParams &kp, int mode, float *out,
               const float *ybase, const float *ydelta, const float *qa,
               const float *qb, float *q_io, const ImpArgs *imp = nullptr);

@@ -397,9 +397,6 @@ __device__ __forceinline__ void fin_grad(const KParams &kp, const FinArgs &A, co
     double v[3] = {dec, dmax, ymax}, o[3];
     const bool mx[3] = {false, true, true};
     if (grid_reduce<3, NT, PB * D>(v, mx, A.red, A.ticket, o)) {
-      A.scal[SC_DEC] = o[0] / (double)kp.N;
-      A.scal[SC_DMAX] = o[1];
-      A.scal[SC_YMAX] = o[2];
       if (!(fabs(o[0]) <= 1e300)) vds_flag(A.err, VDS_ENAN);
       if (A.imp.st) imp_after_grad(A.imp.st, o[0] / (double)kp.N, o[1], o[2], A.err);
     }

@@ -216,25 +216,16 @@ __global__ void __launch_bounds__(NT)
 
 // --------------------------------------------------------------- prep kernel
 
+// Records of the N x D points y, and far ones up to Npad.
 template <int D>
-__global__ void k_prep(int N, int Npad, float c, const float *__restrict__ base,
-                       const float *__restrict__ delta, const float *__restrict__ dir,
-                       float alpha, float *__restrict__ delta_out, float *__restrict__ rec) {
+__global__ void k_prep(int N, int Npad, float c, const float *__restrict__ y, float *__restrict__ rec) {
   constexpr int DP = Rec<D>::DP;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Npad) return;
   float o[DP];
   if (i < N) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      float dl = 0.f;
-      if (delta) {
-        dl = delta[(size_t)i * D + d];
-        if (dir) dl = dl - alpha * dir[(size_t)i * D + d];
-        if (delta_out) delta_out[(size_t)i * D + d] = dl;
-      }
-      o[d] = c * (base[(size_t)i * D + d] + dl);
-    }
+    for (int d = 0; d < D; ++d) o[d] = c * y[(size_t)i * D + d];
   } else {
 #pragma unroll
     for (int d = 0; d < D; ++d) o[d] = VDS_PAD_COORD;
@@ -242,7 +233,7 @@ __global__ void k_prep(int N, int Npad, float c, const float *__restrict__ base,
 #pragma unroll
   for (int d = D; d < DP; ++d) o[d] = 0.f;
   if constexpr (HasNorm<D>::value) {
-    // the squared norm, rounded as the expanded density pass forms x.x
+    // the squared norm, rounded as the tensor-core passes subtract it
     float nrm = o[0] * o[0];
 #pragma unroll
     for (int d = 1; d < D; ++d) nrm = fmaf(o[d], o[d], nrm);
@@ -327,8 +318,7 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) *ticket = 0u;
 }
 
-// Record of y (scaled by c, w = 0, the norm where there is room), or of a
-// padding row.
+// Record of y (scaled by c, everything behind it zero), or of a padding row.
 template <int D>
 __device__ __forceinline__ void put_record(float *rec, int i, float c, const float (&y)[D], bool pad) {
   constexpr int DP = Rec<D>::DP;
@@ -456,12 +446,10 @@ int launch_pair(vds_ctx *c, int N, Sched &sc, int Ni, const float *reci, const I
 }
 
 template <int D>
-int prep_impl(vds_ctx *c, const KParams &kp, const float *base, const float *delta,
-              const float *dir, float alpha, float *delta_out) {
+int prep_impl(vds_ctx *c, const KParams &kp, const float *y) {
   const int Npad = (kp.N + TJ - 1) / TJ * TJ;
   VDS_TRY(vds_ensure(c, c->rec, (size_t)Npad * Rec<D>::DP * sizeof(float)));
-  k_prep<D><<<(Npad + 255) / 256, 256, 0, c->stream>>>(kp.N, Npad, kp.c, base, delta, dir, alpha,
-                                                       delta_out, (float *)c->rec.ptr);
+  k_prep<D><<<(Npad + 255) / 256, 256, 0, c->stream>>>(kp.N, Npad, kp.c, y, (float *)c->rec.ptr);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   return VDS_OK;
@@ -648,8 +636,8 @@ int launch_small_shape(vds_ctx *c, const KParams &kp, const FinArgs &A) {
 // 256; N = 1536, D = 9 19.7 / 18.8.
 template <int D, int MODE>
 int launch_small(vds_ctx *c, const KParams &kp, const FinArgs &A) {
-  constexpr int RI1_N = D <= 10 ? 2432 : 1216, RI2 = D >= 8 && D <= 10 ? 4 : 2;
-  if (kp.N > RI1_N) return launch_small_shape<D, MODE, RI2, (8 * RI2 * D > 512 ? 1024 : 512)>(c, kp, A);
+  constexpr int RI2 = D >= 8 && D <= 10 ? 4 : 2;
+  if (kp.N > (D <= 10 ? 16 : 8) * c->num_sms) return launch_small_shape<D, MODE, RI2, 512>(c, kp, A);
   if (D <= 3 || kp.N <= 8 * c->num_sms) return launch_small_shape<D, MODE, 1, 1024>(c, kp, A);
   return launch_small_shape<D, MODE, 1, 512>(c, kp, A);
 }
@@ -721,11 +709,10 @@ __global__ void __launch_bounds__(NT_FIN)
 
 template <int D>
 int query_impl(vds_ctx *c, const KParams &kp, const float *q, const float *y, int M, float *f_out) {
-  VDS_TRY(prep_impl<D>(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(prep_impl<D>(c, kp, q));
   const int Mpad = (M + TJ - 1) / TJ * TJ;
   VDS_TRY(vds_ensure(c, c->recq, (size_t)Mpad * Rec<D>::DP * sizeof(float)));
-  k_prep<D><<<(Mpad + 255) / 256, 256, 0, c->stream>>>(M, Mpad, kp.c, y, nullptr, nullptr, 0.f, nullptr,
-                                                       (float *)c->recq.ptr);
+  k_prep<D><<<(Mpad + 255) / 256, 256, 0, c->stream>>>(M, Mpad, kp.c, y, (float *)c->recq.ptr);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
   PartSrc src;
@@ -795,7 +782,7 @@ int rows_records(vds_ctx *c, int row0, int nrows) {
 // rho of the rows (FP32) from the density pass over all N columns.
 template <int D>
 int rows_density_impl(vds_ctx *c, const KParams &kp, const float *q, int row0, int nrows, float *rho_rows) {
-  VDS_TRY(prep_impl<D>(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(prep_impl<D>(c, kp, q));
   VDS_TRY(rows_records<D>(c, row0, nrows));
   PartSrc src;
   VDS_TRY((launch_pass<D, false>(c, kp.N, src.sc, nrows, (const float *)c->recq.ptr)));
@@ -813,7 +800,7 @@ int rows_density_impl(vds_ctx *c, const KParams &kp, const float *q, int row0, i
 template <int D>
 int rows_grad_impl(vds_ctx *c, const KParams &kp, const float *q, const float *rho, int row0, int nrows,
                    int mode, float *out) {
-  VDS_TRY(prep_impl<D>(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(prep_impl<D>(c, kp, q));
   k_set_w<D><<<(kp.N + 255) / 256, 256, 0, c->stream>>>(kp.N, rho, (float *)c->rec.ptr, c->err);
   VDS_CUDA_TRY(cudaGetLastError());
   ++c->launches;
@@ -874,9 +861,8 @@ int imp_trial_impl(vds_ctx *c, const KParams &kp, const ImpArgs &imp, const floa
 // One translation unit per supported D (pair_d<D>.cu) instantiates the passes
 // through this macro, so the library builds in parallel.
 #define VDS_PAIR_INSTANTIATE(DD)                                                              \
-  int vds_prep_##DD(vds_ctx *c, const KParams &kp, const float *base, const float *delta,     \
-                    const float *dir, float alpha, float *delta_out) {                        \
-    return vds_pair::prep_impl<DD>(c, kp, base, delta, dir, alpha, delta_out);                \
+  int vds_prep_##DD(vds_ctx *c, const KParams &kp, const float *y) {                          \
+    return vds_pair::prep_impl<DD>(c, kp, y);                                                 \
   }                                                                                           \
   int vds_density_##DD(vds_ctx *c, const KParams &kp, float *rho_out, bool want_energy,       \
                        const float *ybase, const float *ydelta, const float *qa,              \

@@ -20,11 +20,12 @@ namespace vds_pair {
 
 constexpr int SM_DENS = -1;  // MODE of the density pass; a GradMode otherwise
 // Least CTAs per SM (0: the compiler's own register budget), by what was faster
-// for a dimension with two chains: N = 4800, D = 2 28.0 -> 22.8 us a step, D = 9
-// 57 -> 51, D = 10 69 -> 58; N = 6000, D = 4 58 -> 52 (one chain: 22.9, 52, 67, 46).
-constexpr int sm_minb(int D, int RI, bool dens) {
-  if (RI == 1) return 0;
-  if (D <= 3 || (D >= 8 && D <= 10)) return 1;
+// for a dimension: with two chains N = 4800, D = 2 28.0 -> 22.8 us a step, D = 9
+// 57 -> 51, D = 10 69 -> 58; N = 6000, D = 4 58 -> 52 (one chain: 22.9, 52, 67, 46);
+// five implicit steps of N = 512, D = 2 687 -> 645 us (32 registers by itself).
+constexpr int sm_minb(int D, int RI, int NT, bool dens, bool imp) {
+  if (RI == 1) return imp && NT == 1024 && D <= 9 ? 1 : 0;
+  if (D == 2 || (D == 3 && !imp) || (D >= 8 && D <= 10)) return 1;
   return D == 4 && !dens ? 3 : D == 16 && dens ? 2 : 0;
 }
 // From here on (16 warps: 48 records a lane) a lane's records go in two chains,
@@ -34,7 +35,7 @@ constexpr int sm_minb(int D, int RI, bool dens) {
 constexpr int SM_TWO_N = 3073;
 
 template <int D, int S, int RI, int NT, int MODE>
-__global__ void __launch_bounds__(NT, sm_minb(D, RI, MODE == SM_DENS)) k_small(const float *rec, KParams kp, FinArgs A) {
+__global__ void __launch_bounds__(NT, sm_minb(D, RI, NT, MODE == SM_DENS, MODE == GM_IMPLICIT_DIR)) k_small(const float *rec, KParams kp, FinArgs A) {
   constexpr bool GRAD = MODE != SM_DENS;
   constexpr int DP = Rec<D>::DP, ACC = GRAD ? D : 1, PB = 8 * RI, W = NT / 32;
   constexpr int V = (D + (GRAD ? 1 : 0) + 3) / 4;

@@ -8,7 +8,7 @@
 //   gradient  u = khat (w_I + w_J), S_I += u dq, S_J -= u dq:   4D + 2 and one
 //             ex2 (2 (3D + 2) and two ex2).
 // The FP32 pipe bounds both passes, as it bounds the ordered form (k_pair).
-// N = 65536, D = 9: density 2.46 -> 1.40 ms, gradient 3.86 -> 2.98 ms (ordered
+// N = 65536, D = 9: density 2.46 -> 1.36 ms, gradient 3.86 -> 2.93 ms (ordered
 // form -> this one); N = 16384, D = 3: 78 -> 51 and 128 -> 88 us.
 //
 // i-tiles of TI = NT x RI particles, j-chunks of TJS; tile t takes the chunks
@@ -22,7 +22,7 @@
 // shared-memory traffic of a step (records, and the D sums in and out) is paid
 // once per RI pairs of a lane.
 //
-// Sums: the i side in FP32 over 64 records (large gradient tiles: 128),
+// Sums: the i side in FP32 over 64 records,
 // Kahan-compensated in shared memory across them; the j side in FP32 over the
 // RI particles of a step, then over the 32 steps of a warp (one chain of 32 RI
 // terms would save D of its 4D RI operations a step, 3 % of a pass, and double
@@ -97,7 +97,7 @@ __device__ __forceinline__ void sym_run(const float *__restrict__ rec, int N, in
   // against 1.13e-7 (and k_pair's 1.13e-7)
   constexpr int FOLD = 64 / TJS;
   using JS = JSlots<ACC, TJS>;
-  static_assert(TI % TJS == 0 && TJS % 32 == 0 && 256 % TJS == 0, "tile shapes");
+  static_assert(TI % TJS == 0 && TJS % 32 == 0 && 64 % TJS == 0, "tile shapes");
   float4 *tile = reinterpret_cast<float4 *>(sm_raw);                   // [2][V][TJS]
   float *js = reinterpret_cast<float *>(sm_raw + L::TILE);             // [2][W][ACC x TJS]
   float *ks = reinterpret_cast<float *>(sm_raw + L::TILE + L::JS);     // [RI x ACC][NT] sums

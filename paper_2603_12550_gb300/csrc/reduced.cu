@@ -486,7 +486,7 @@ int density_1e4(vds_ctx *c, const KParams &kp, const float *qt) {
 int brownian_dev(vds_ctx *c, const pod_basis *b, const float *P, int N, int D, const KParams &kp,
                  float *qt, float *U1, float *U2, double *G1, double *G2) {
   VDS_TRY(pod_lift_dev(c, b, P, N, D, qt));
-  VDS_TRY(pass_prep(c, kp, qt, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(pass_prep(c, kp, qt));
   // the density at the lifted state feeds only the frozen terms (X^B within
   // 1e-4 of the FP64 oracle)
   VDS_TRY(density_1e4(c, kp, qt));
@@ -565,7 +565,7 @@ int pod_step(vds_ctx *c, const pod_basis *b, float *P, int N, int D, const vds_p
   } else {
     for (int n0 = 0; n0 < nsteps; ++n0) {
       VDS_TRY(pod_lift_dev(c, b, P, N, D, qt));
-      VDS_TRY(pass_prep(c, kp, qt, nullptr, nullptr, 0.f, nullptr));
+      VDS_TRY(pass_prep(c, kp, qt));
       VDS_TRY(pass_density(c, kp, nullptr, false, qt, nullptr, nullptr, nullptr));
       VDS_TRY(pass_grad(c, kp, GM_VEL, vel, qt, nullptr, nullptr, nullptr, nullptr));
       VDS_TRY(pod_project_dev(c, b, vel, N, D, Pdot, nullptr));
@@ -698,7 +698,7 @@ int pod_step_score(vds_ctx *c, const pod_basis *b, vds_score *sc, float *P, int 
       // full density (every 1/rho_J enters S_I), gradient of the checked rows;
       // the density within about 1e-4 (against a check threshold of order 0.1
       // and a fallback step held to 1e-3)
-      VDS_TRY(pass_prep(c, kS, qt, nullptr, nullptr, 0.f, nullptr));
+      VDS_TRY(pass_prep(c, kS, qt));
       VDS_TRY(density_1e4(c, kS, qt));
       // compact exact S of the checked rows (after the FP64 segment partials)
       // in the shared scratch, taken afresh at every check

@@ -295,7 +295,7 @@ int vds_energy_grad(vds_ctx *c, const float *q, int N, int D, const vds_params *
   DeviceGuard dg(c->device);
   const KParams kp = make_kparams(p, N, D);
   const float *qa = q_star ? q : nullptr;
-  VDS_TRY(pass_prep(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(pass_prep(c, kp, q));
   VDS_TRY(pass_density(c, kp, rho, E != nullptr, q, nullptr, qa, q_star));
   if (g) VDS_TRY(pass_grad(c, kp, GM_OUT, g, q, nullptr, qa, q_star, nullptr));
   if (E) {
@@ -334,7 +334,7 @@ int vds_density_tc(vds_ctx *c, const float *q, int N, int D, const vds_params *p
   if (D != 6 && D != 9) return VDS_EARG;
   DeviceGuard dg(c->device);
   const KParams kp = make_kparams(p, N, D);
-  VDS_TRY(pass_prep(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(pass_prep(c, kp, q));
   return pass_density_tc(c, kp, rho);
 }
 
@@ -355,7 +355,7 @@ int vds_density_at(vds_ctx *c, const float *q, int N, int D, const vds_params *p
 // timing on (its events belong to single launches), or if the capture fails,
 // the steps are launched one by one, as is an odd last one.
 static int step_explicit(vds_ctx *c, float *q, const KParams &kp, int nsteps) {
-  VDS_TRY(pass_prep(c, kp, q, nullptr, nullptr, 0.f, nullptr));
+  VDS_TRY(pass_prep(c, kp, q));
   auto one_step = [&]() -> int {
     VDS_TRY(pass_density(c, kp, nullptr, false, q, nullptr, nullptr, nullptr));
     return pass_grad(c, kp, GM_EXPLICIT, nullptr, q, nullptr, nullptr, nullptr, q);

@@ -61,6 +61,38 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// Packed pairs of FP32 values (f32x2 instructions: one issue slot for two
+// lanes' worth of FP32 work, each half rounded as the scalar instruction).
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(unsigned long long v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ uint64_t global_timer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -242,6 +274,6 @@ int vds_time_end(vds_ctx *c, int pk);
 int vds_sync_status(vds_ctx *c);  // synchronise the stream, read+clear err
 
 // Scalar slots in ctx->scal
-enum { SC_E = 0, SC_DEC = 1, SC_DMAX = 2, SC_YMAX = 3, SC_H = 4, SC_AUX = 5, SC_COUNT = 320 };
+enum { SC_E = 0, SC_H = 4, SC_AUX = 5, SC_COUNT = 320 };
 // Ticket slots
 enum { TK_DENS = 0, TK_GRAD = 1, TK_STRESS = 2, TK_MISC = 3, TK_COLSUM = 8 /* .. 15 */, TK_COUNT = 16 };
