@@ -10,6 +10,9 @@ fused Euler update of all particles -- through the public C ABI (vds_step).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
+The result is one JSON line on stdout; the secondary measurements (extras) are
+one on stderr.
+
 N > 1 (launched by torchrun, one rank per GPU) splits the one cloud by
 particle rows over the ranks: each rank evaluates its rows against all
 particles, with two NCCL all-gathers per step (strong scaling; the job's
@@ -123,6 +126,24 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
+def _rounded(x):
+    """Floats to seven significant digits, through lists and dicts."""
+    if isinstance(x, float):
+        return float(f"{x:.7g}")
+    if isinstance(x, dict):
+        return {k: _rounded(v) for k, v in x.items()}
+    return [_rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def report(line, extras=None):
+    """The result as one short JSON line on stdout (what is kept of a run's
+    output may be its last 3000 characters); the extras as one of their own on
+    stderr."""
+    if extras is not None:
+        print(json.dumps({"extras": _rounded(extras)}), file=sys.stderr, flush=True)
+    print(json.dumps(_rounded(line)), flush=True)
+
+
 def _peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -230,7 +251,7 @@ def run_reference(a, wl, rank):
             "cpu_baseline": {"value": value, "unit": UNIT, "cores": cores, "kind": "oracle",
                              "sample": sample_txt},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    report(line)
 
 
 def _extras(ctx, vds, inputs, torch, wl, h, stream, which):
@@ -926,7 +947,7 @@ def run_sharded(a, wl, rank, world, local, dist):
             "e2e": {"value": a.steps / (e2e_ms / 1e3), "unit": UNIT, "h2d_bytes_per_step": int(q0.nbytes),
                     "d2h_bytes_per_step": int(st.C * D * 4)},
             "gpu_launches": int(launches), "clocks": clocks, "roofline": roof, "cpu_baseline": None}
-    print(json.dumps(line), flush=True)
+    report(line)
 
 
 def main():
@@ -1085,8 +1106,8 @@ def main():
             "config": _config(wl, h),
             "pair_interactions_per_s": value * N * N,
             "e2e": e2e, "gpu_launches": int(launches), "clocks": clocks, "roofline": roof,
-            "cpu_baseline": cpu, "extras": extras}
-    print(json.dumps(line), flush=True)
+            "cpu_baseline": cpu}
+    report(line, extras)
     if dist:
         dist.destroy_process_group()
 
