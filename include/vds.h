@@ -21,7 +21,7 @@
  *    over unordered pairs (about N^2 / 4608 x 8 D bytes for N >= 49152, three times
  *    that below, at most 4 GiB: 67 MB at N = 65536, D = 9), of the tensor-core
  *    density (N^2 / 128 bytes, at most 1 GiB) and the keys of the median
- *    bandwidth (at most 1 GiB: 63 MB at N = 65536), up to a quarter more each
+ *    bandwidth (at most 4 GiB: 63 MB at N = 65536), up to a quarter more each
  *    as room to grow.  The first and the last are taken only within a quarter
  *    of the memory that is free on the device at that time, the second in
  *    smaller pieces where it cannot be had; the calls work without them, more
@@ -92,7 +92,9 @@ VDS_API const char *vds_strerror(int status);
 /* Kernel bandwidth (Sec. 2.2).  rule 0: median rule of Eq. model_bandwidth,
  * h = med_{J<K} |q_J - q_K| / sqrt(2 ln N), med the lower middle order
  * statistic of the N(N-1)/2 distances (exact selection on FP32 squared
- * distances).  rule 1: Silverman, h = sigma (4/((D+2)N))^(1/(D+4)) with sigma
+ * distances; clouds of many equal distances, of particles hundreds of times
+ * farther out than the rest, or of more than about three million particles take
+ * about ten times as long).  rule 1: Silverman, h = sigma (4/((D+2)N))^(1/(D+4)) with sigma
  * the mean per-coordinate sample standard deviation.  N >= 2.  *h: host. */
 VDS_API int vds_bandwidth(vds_ctx *ctx, const float *q, int N, int D, int rule,
                   double *h);

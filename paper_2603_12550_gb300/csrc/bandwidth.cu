@@ -13,7 +13,7 @@
 // Where the bracket misses the median (by the counts of step 2; once in 10^6
 // clouds), or the sample shows many equal distances, or a particle lies so far
 // out that the screen of step 2 has no resolution, or the keys take more room
-// than there is (from about a million particles on), a radix select by three
+// than there is (from about three million particles on), a radix select by three
 // histogram passes over all pairs (k_hist) takes over.  Clouds of up to SMALL_PAIRS
 // pairs write all keys and select among them.
 //
@@ -140,7 +140,7 @@ __global__ void k_sel_digit(SelState *st, unsigned long long *ghist, int pass, l
 // ------------------------------------------------- bracketed selection
 
 constexpr unsigned long long SMALL_PAIRS = 1ull << 22;
-constexpr unsigned long long MOST_KEYS = 1ull << 28;  // 1 GiB of workspace: clouds of about a million particles
+constexpr unsigned long long MOST_KEYS = 1ull << 30;  // 4 GiB of workspace: clouds of about three million particles
 constexpr int SEL_NT = 512, SEL_BINS = 2048, SEL_BITS = 11;
 
 // Selection of up to two order statistics among keys in [lo, hi], by digits of
